@@ -49,7 +49,7 @@ typedef struct stencil_grid* stencil_t; /* opaque, owned by the library */
 
 enum stencil_kind { STENCIL_7PT_CONST = 0, STENCIL_7PT_VAR = 1, STENCIL_25PT_VAR = 2 };
 enum stencil_dtype { STENCIL_F32 = 0, STENCIL_F64 = 1, STENCIL_BF16 = 2 };
-enum stencil_scheme { STENCIL_PLAIN = 0, STENCIL_BLOCKED = 1, STENCIL_AUTO = 2, STENCIL_WAVEFRONT = 3 };
+enum stencil_scheme { STENCIL_PLAIN = 0, STENCIL_BLOCKED = 1, STENCIL_AUTO = 2, STENCIL_WAVEFRONT = 3, STENCIL_OVERLAP = 4 };
 /* Where a dense array passed to set_coeffs / set_field / get_field lives.
  * STENCIL_HOST: host memory; the call waits for its copy when the caller needs
  * the data back (page-locked memory is moved by the library's copy kernel,
@@ -163,9 +163,15 @@ int stencil_set_field(stencil_t h, const void* src, double halo_value, int where
  * STENCIL_EINVAL; bit-identical to the plain sweep), or
  * STENCIL_BLOCKED with *tuning (NULL: library default: D_w = 8R, N_F = 2 where it
  * fits (1 for the 7-point variable stencil with FP32 coefficients), 16 warps for
- * R = 1, the widest x tile whose rows fit one warp of vectors), or
+ * R = 1, the widest x tile whose rows fit one warp of vectors),
+ * STENCIL_OVERLAP (7-point stencils with an FP32 field, else STENCIL_EINVAL: overlapped tiles
+ * that each advance three steps per pass with their planes in registers, all passes of a run in
+ * one persistent launch with bounded waits; needs a bound workspace; tuning->nf = z chunks per
+ * column of tiles, 0 or NULL: chosen from the grid and the GPU; other fields ignored;
+ * bit-identical to the plain sweep), or
  * STENCIL_AUTO (plain for FP64 fields and the 25-point stencil, where the plain sweep
- * measured faster on GB300; else the default blocked tuning when it fits, else plain).
+ * measured faster on GB300; overlapped tiles for the 7-point stencils in FP32; without a
+ * workspace the default blocked tuning when it fits, else plain).
  * Returns STENCIL_ENOSMEM / STENCIL_EINVAL for an infeasible blocked tuning. */
 int stencil_set_tuning(stencil_t h, int scheme, const stencil_tuning* tuning);
 

@@ -26,6 +26,7 @@ struct stencil_grid {
     BlockedTune tune;
     WaveTune wtune;
     int plain_prefetch;  // plain sweep's prefetch depth (0 or 2)
+    int overlap_chunks;  // overlapped sweep's z chunks (0: chosen per run)
     bool tune_set;
     long long launches;
     long long tile_passes;  // wavefront passes run with tile copies into shared memory
@@ -166,6 +167,7 @@ int stencil_create(stencil_t* out, int kind, int nx, int ny, int nz, int field_d
     h->parity = 0;
     h->scheme = STENCIL_PLAIN;
     h->tune_set = false;
+    h->overlap_chunks = 0;
     h->launches = 0;
     h->tile_passes = 0;
     h->halo_ok = false;
@@ -345,12 +347,26 @@ int stencil_set_tuning(stencil_t h, int scheme, const stencil_tuning* tuning) {
         h->wtune = w;
         return STENCIL_OK;
     }
+    if (scheme == STENCIL_OVERLAP) {
+        if (!overlap_ok(args_of(h)) || !h->ws) return STENCIL_EINVAL;
+        if (tuning && (tuning->nf < 0 || tuning->nf > h->L.nz)) return STENCIL_EINVAL;
+        h->scheme = STENCIL_OVERLAP;
+        h->overlap_chunks = tuning ? tuning->nf : 0;
+        return STENCIL_OK;
+    }
     if (scheme != STENCIL_BLOCKED && scheme != STENCIL_AUTO) return STENCIL_EINVAL;
     if (scheme == STENCIL_AUTO && (h->fdt == DT_F64 || h->kind == STENCIL_25PT_VAR)) {
         // Measured on GB300: FP64 sweeps are bound by the FP64 units (1/60 of the FP32 rate),
         // where the blocked sweep's x-tile overlap only adds work, and the 25-point rings fit
         // only narrow x tiles; the plain sweep is faster for both.
         h->scheme = STENCIL_PLAIN;
+        return STENCIL_OK;
+    }
+    if (scheme == STENCIL_AUTO && overlap_ok(args_of(h)) && h->ws) {
+        // The 7-point stencils in FP32: faster than the plain sweep and the diamonds at every size
+        // measured, 64^3 to 1024^3 (overlap_impl.cuh has the figures).
+        h->scheme = STENCIL_OVERLAP;
+        h->overlap_chunks = 0;
         return STENCIL_OK;
     }
     BlockedTune t = default_tune(h);
@@ -379,7 +395,7 @@ int stencil_run(stencil_t h, int T) {
     if (!h->bound) return STENCIL_EUNBOUND;
     if (T == 0) return STENCIL_OK;
     SweepArgs a = args_of(h);
-    if ((h->scheme == STENCIL_BLOCKED || h->scheme == STENCIL_WAVEFRONT) && h->ws && !h->status_armed) {
+    if (h->scheme != STENCIL_PLAIN && h->ws && !h->status_armed) {
         if (cudaMemsetAsync(static_cast<int*>(h->ws) + PERSIST_WS_STATUS, 0, sizeof(int), h->stream) != cudaSuccess)
             return STENCIL_ECUDA;
         h->status_armed = true;
@@ -388,6 +404,22 @@ int stencil_run(stencil_t h, int T) {
         cudaError_t e = wave_run(a, h->field, h->parity, T, h->wtune, h->ws, GRID_WORKSPACE_BYTES, h->ctl, h->stream,
                                  &h->launches, &h->tile_passes);
         if (e == cudaErrorInvalidValue) return STENCIL_EINVAL;
+        if (e != cudaSuccess) return STENCIL_ECUDA;
+    } else if (h->scheme == STENCIL_OVERLAP) {
+        cudaError_t e = overlap_run(a, h->field, h->parity, T, h->overlap_chunks, static_cast<int*>(h->ws),
+                                    GRID_WORKSPACE_BYTES, h->ctl, h->stream, &h->launches);
+        if (e == cudaErrorNotReady) {
+            // too many items for one launch: in two parts, or by plain steps
+            if (T > 6) {
+                int rc = stencil_run(h, T / 2);
+                return rc != STENCIL_OK ? rc : stencil_run(h, T - T / 2);
+            }
+            e = cudaSuccess;
+            for (int t = 0; t < T && e == cudaSuccess; ++t, ++h->launches) {
+                const int p = (h->parity + t) & 1;
+                e = plain_step(a, h->field[p], h->field[p ^ 1], h->stream);
+            }
+        }
         if (e != cudaSuccess) return STENCIL_ECUDA;
     } else if (h->scheme == STENCIL_BLOCKED) {
         cudaError_t e = cudaErrorNotReady;

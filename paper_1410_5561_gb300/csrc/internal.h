@@ -118,6 +118,13 @@ cudaError_t wave_run(const SweepArgs& a, void* const field[2], int p0, int T, co
 cudaError_t wave_tma_pass(const SweepArgs& a, void* const* levels, int h, const WaveTune& tn, int* ws,
                           const PersistCtl& ctl, cudaStream_t st, long long* launches);
 
+// T steps by overlapped tiles in one persistent launch (overlap.cu; overlap_ok: the 7-point
+// stencils with an FP32 field). chunks: z chunks per column of tiles (0: chosen from the grid and
+// the GPU). cudaErrorNotReady: more tiles than the workspace has counters for.
+bool overlap_ok(const SweepArgs& a);
+cudaError_t overlap_run(const SweepArgs& a, void* const field[2], int p0, int T, int chunks, int* ws, size_t ws_bytes,
+                        const PersistCtl& ctl, cudaStream_t st, long long* launches);
+
 // Shared-memory bytes the blocked kernel needs for a tuning (0 if infeasible).
 size_t blocked_smem_bytes(const SweepArgs& a, const BlockedTune& tune);
 

@@ -9,7 +9,13 @@
 #include <cuda.h>
 #include <stdint.h>
 
+#include "common.cuh"
+
 namespace stg {
+
+// Tensor map of a padded array of one grid (eb bytes per element) with boxes of (bx, by, 1)
+// elements; false if the driver refuses it. Defined in wave_tma.cu.
+bool tma_encode_3d(CUtensorMap* m, CUtensorMapDataType dt, int eb, const void* base, const Layout& L, int bx, int by);
 
 constexpr unsigned TMA_WAIT_POLLS = 1u << 22;  // with the back-off below: > 0.25 s
 

@@ -305,7 +305,9 @@ PFN_cuTensorMapEncodeTiled_v12000 tma_encoder() {
     return fn;
 }
 
-bool encode_3d(CUtensorMap* m, CUtensorMapDataType dt, int eb, const void* base, const Layout& L, int bx, int by) {
+}  // namespace
+
+bool tma_encode_3d(CUtensorMap* m, CUtensorMapDataType dt, int eb, const void* base, const Layout& L, int bx, int by) {
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tma_encoder();
     if (!enc) return false;
     const cuuint64_t dims[3] = {(cuuint64_t)L.px, (cuuint64_t)L.py, (cuuint64_t)L.pz};
@@ -316,6 +318,8 @@ bool encode_3d(CUtensorMap* m, CUtensorMapDataType dt, int eb, const void* base,
                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+namespace {
 
 template <typename TC>
 cudaError_t wave_tma_t(const SweepArgs& a, void* const* lvl, int h, const WaveTune& tn, int* ws, const PersistCtl& ctl,
@@ -340,9 +344,9 @@ cudaError_t wave_tma_t(const SweepArgs& a, void* const* lvl, int h, const WaveTu
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kfn, 32 * (TW_BY + 1), Cfg::SMEM))) return e;
     if (ctas > (long long)per * sms) return cudaErrorNotReady;  // every (level, tile) CTA must be resident
     TwArgs A{};
-    if (!encode_3d(&A.fmap[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, lvl[0], L, TW_XW, TW_BY + 2 * TW_R))
+    if (!tma_encode_3d(&A.fmap[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, lvl[0], L, TW_XW, TW_BY + 2 * TW_R))
         return cudaErrorNotReady;
-    if (!encode_3d(&A.fmap[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h > 1 ? lvl[1] : lvl[0], L, TW_XW,
+    if (!tma_encode_3d(&A.fmap[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h > 1 ? lvl[1] : lvl[0], L, TW_XW,
                    TW_BY + 2 * TW_R))
         return cudaErrorNotReady;
     for (int m = 0; m < 13; ++m) A.cf[m] = a.coef[m];

@@ -1,0 +1,74 @@
+"""Overlapped-tile sweep against the plain sweep, bit for bit (the same operations on the same
+operands in the same order), at the edges of its tiles: rows of one vector to several tiles, row
+counts around the tile heights of the three instantiations, z chunks thinner and thicker than the
+overlap, step counts with and without a remainder; and against the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from tests._util import Problem, step_tol
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(1, 1, 1), (3, 5, 2), (4, 32, 7), (5, 33, 3), (124, 60, 9), (125, 61, 12), (128, 31, 40), (129, 17, 5),
+          (248, 30, 11), (249, 44, 4), (252, 12, 26), (131, 13, 23), (376, 9, 8), (64, 89, 19)]
+KINDS = [("7pt_const", None), ("7pt_var", None), ("7pt_var", "bf16")]
+
+
+def _pair(kind, cdt, shape, T, chunks, seed=51):
+    import torch
+    from paper_1410_5561_gb300.stencil import Tuning
+    p = Problem(kind, *shape, fdt="f32", cdt=cdt, seed=seed, halo=-0.625)
+    a, b = p.make(), p.make()
+    a.set_tuning("plain")
+    b.set_tuning("overlap", Tuning(6, chunks, 0, 0))
+    a.run(T)
+    b.run(T)
+    b.sync()
+    assert a.parity == b.parity
+    assert torch.equal(a.current, b.current)
+    b.current.fill_(-0.625)  # what is left of the array is its halo, untouched
+    assert bool((b.fields[b.parity] == -0.625).all())
+    return p, a
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("kind,cdt", KINDS)
+def test_overlap_is_bitwise_equal_to_plain(kind, cdt, shape):
+    for chunks in (0, 1, min(3, shape[2])):
+        _pair(kind, cdt, shape, 3, chunks)
+    _pair(kind, cdt, shape, 7, 0)
+
+
+@pytest.mark.parametrize("kind,cdt", KINDS)
+def test_overlap_larger_grid_and_oracle(kind, cdt):
+    T = 20
+    p, a = _pair(kind, cdt, (301, 107, 75), T, 0)
+    ref = p.oracle(T)
+    got = a.get_field().double().cpu().numpy()
+    assert oracle.step_normalised_l2(got, ref, T) <= step_tol("f32")
+    assert np.max(np.abs(got - ref)) <= p.elementwise_tol(T)
+
+
+def test_overlap_is_captured_in_a_graph():
+    import torch
+    p = Problem("7pt_var", 140, 50, 33, fdt="f32", seed=5, halo=0.25)
+    a, b = p.make(), p.make()
+    a.set_tuning("plain")
+    b.set_tuning("overlap")
+    g = b.capture(8)
+    g.replay()
+    g.replay()
+    a.run(16)
+    torch.cuda.synchronize()
+    assert torch.equal(a.current, b.current)
+
+
+def test_overlap_refuses_other_stencils():
+    from paper_1410_5561_gb300.stencil import Stencil, Tuning
+    import torch
+    for kind, dt in (("25pt_var", torch.float32), ("7pt_const", torch.float64)):
+        with pytest.raises(Exception):
+            Stencil(kind, 20, 20, 20, dtype=dt).set_tuning("overlap")
+    with pytest.raises(Exception):
+        Stencil("7pt_const", 20, 20, 20).set_tuning("overlap", Tuning(6, 21, 0, 0))
