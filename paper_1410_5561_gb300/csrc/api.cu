@@ -284,8 +284,18 @@ int stencil_set_coeffs(stencil_t h, const double* scalars, const void* const* ar
     if (!arrays) return STENCIL_EINVAL;
     int nc = kind_ncoef(h->kind);
     int eb = dtype_bytes(h->cdt);
+    const void* view[13];
+    bool direct = true;
     for (int m = 0; m < nc; ++m) {
         if (!arrays[m]) return STENCIL_EINVAL;
+        direct = direct && (view[m] = device_view(arrays[m])) != nullptr;
+    }
+    if (direct) {
+        if (pack_rows(h->L, eb, view, h->coef, nc, h->stream) != cudaSuccess) return STENCIL_ECUDA;
+        ++h->launches;
+        return STENCIL_OK;
+    }
+    for (int m = 0; m < nc; ++m) {
         cudaError_t e = fill_value(h->coef[m], h->L.count(), h->cdt, 0.0, h->stream);
         if (e != cudaSuccess) return STENCIL_ECUDA;
         ++h->launches;

@@ -47,6 +47,8 @@ cudaError_t fill_value(void* p, size_t n, int dt, double v, cudaStream_t s);
 cudaError_t dense_copy(void* dst, const void* src, size_t bytes, int ctas, cudaStream_t s);
 // Dense interior rows <-> padded layout (src/dst device or device-mapped host pointers).
 cudaError_t copy_rows(const Layout& L, int eb, const void* src, void* dst, bool to_padded, cudaStream_t s);
+// n (at most 13) dense arrays into padded ones, zeros in every other cell (pointers as above).
+cudaError_t pack_rows(const Layout& L, int eb, const void* const* src, void* const* dst, int n, cudaStream_t s);
 
 // Temporally blocked run of T steps from parity p0 (array (p0 + t) & 1 holds u_t).
 // Returns cudaErrorInvalidValue for an infeasible tuning, after checking it on the host.
