@@ -49,19 +49,55 @@ struct AdjSteps {
     const TF* u[ADJ_GROUP];
 };
 
-template <int KIND, typename TF, int BY>
-__global__ void __launch_bounds__(32 * BY) adjoint_grad_kernel(Layout L, AdjSteps<TF> S, int nsteps, AdjGrad G,
-                                                               int zchunk) {
+// FP32 -> FP64 without the FP64 pipe, which also does the hardware conversion and already bounds
+// this kernel: N values at once, by integer operations where all of them are normal numbers (the
+// magnitude times 2^29 as a 64-bit integer is the FP64 significand and exponent field, short of
+// the difference of the two exponent biases), else by the hardware conversion. Exact either way.
+template <int N>
+struct Widen {
+    double d[N];
+    __device__ __forceinline__ explicit Widen(const float* x) {
+        unsigned a[N], lo = 0x7f800000u, hi = 0u;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            a[i] = __float_as_uint(x[i]) & 0x7fffffffu;
+            lo = min(lo, a[i]);
+            hi = max(hi, a[i]);
+        }
+        if (lo >= 0x00800000u && hi < 0x7f800000u) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const unsigned long long w = (unsigned long long)a[i] * (1u << 29) + (896ull << 52);
+                d[i] = __hiloint2double((int)((unsigned)(w >> 32) | (__float_as_uint(x[i]) & 0x80000000u)), (int)(unsigned)w);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < N; ++i) d[i] = (double)x[i];
+        }
+    }
+    __device__ __forceinline__ explicit Widen(const double* x) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) d[i] = x[i];
+    }
+};
+
+// Bound by the FP64 pipe: one fma per coefficient, point and step (14.3 ms at its peak for 13
+// arrays, 256^3, 40 steps). With hardware conversions of the weights on the same pipe it took
+// 34.0 ms, with Widen 19.4, at three CTAs per SM (168 registers, 24 bytes spilled) 17.6; vectors of
+// two points (more warps, but twice the loads) 29.6.
+template <int KIND, typename TF, int V, int NT>
+__global__ void __launch_bounds__(NT, 3) adjoint_grad_kernel(Layout L, AdjSteps<TF> S, int nsteps, AdjGrad G, int zchunk) {
     constexpr int R = KindTraits<KIND>::R;
     constexpr int NC = KindTraits<KIND>::NC;
-    constexpr int V = 16 / sizeof(TF);
     constexpr int J = (R + V - 1) / V;
     constexpr int XL = (2 * J + 1) * V;
     using A = Ar<TF>;
-    const int i0 = (blockIdx.x * 32 + threadIdx.x) * V;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    if (i0 >= L.nx || j >= L.ny) return;
-    const int k0 = blockIdx.z * zchunk;
+    // threads over the plane's vectors in order, so that only its last warp has idle lanes
+    const unsigned nv = (unsigned)(L.nx + V - 1) / V;
+    const unsigned long long q = (unsigned long long)blockIdx.x * NT + threadIdx.x;
+    if (q >= (unsigned long long)nv * (unsigned)L.ny) return;
+    const int j = (int)(q / nv), i0 = (int)(q - (unsigned long long)j * nv) * V;
+    const int k0 = blockIdx.y * zchunk;
     const int k1 = min(L.nz, k0 + zchunk);
     const size_t sy = (size_t)L.px, sz = L.plane();
     const bool full = i0 + V <= L.nx;
@@ -95,24 +131,25 @@ __global__ void __launch_bounds__(32 * BY) adjoint_grad_kernel(Layout L, AdjStep
 #pragma unroll
                 for (int e = 0; e < V; ++e) ux[(q + J) * V + e] = wu.v[e];
             }
-            double lam[V];
-#pragma unroll
-            for (int e = 0; e < V; ++e) lam[e] = (double)lv.v[e];
+            const Widen<V> lam(lv.v);
             // weight of array m: 7-point C0 u(p), C(2a+1) u(p + e_a), C(2a+2) u(p - e_a);
             // 25-point C00 u(p), C(3(d-1)+a+1) (u(p + d e_a) + u(p - d e_a)), the pair sum
             // in the field precision as the forward step forms it
+            {
+                const Widen<V> w(ux + J * V);
 #pragma unroll
-            for (int e = 0; e < V; ++e) gv[0][e] = __fma_rn(lam[e], (double)ux[J * V + e], gv[0][e]);
+                for (int e = 0; e < V; ++e) gv[0][e] = __fma_rn(lam.d[e], w.d[e], gv[0][e]);
+            }
 #pragma unroll
             for (int d = 1; d <= R; ++d) {
+                TF up[3][V], um[3][V];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    TF up[V], um[V];
                     if (a == 0) {
 #pragma unroll
                         for (int e = 0; e < V; ++e) {
-                            up[e] = ux[J * V + e + d];
-                            um[e] = ux[J * V + e - d];
+                            up[a][e] = ux[J * V + e + d];
+                            um[a][e] = ux[J * V + e - d];
                         }
                     } else {
                         const size_t o = (size_t)d * (a == 1 ? sy : sz);
@@ -120,21 +157,32 @@ __global__ void __launch_bounds__(32 * BY) adjoint_grad_kernel(Layout L, AdjStep
                         const Vec<TF, V> vm = ldv_ro<TF, V>(u + p - o);
 #pragma unroll
                         for (int e = 0; e < V; ++e) {
-                            up[e] = vp.v[e];
-                            um[e] = vm.v[e];
+                            up[a][e] = vp.v[e];
+                            um[a][e] = vm.v[e];
                         }
                     }
-                    if constexpr (KIND == K7V) {
-                        // C(2a+1) weighs u(p + e_a), C(2a+2) weighs u(p - e_a)
+                }
+                if constexpr (KIND == K7V) {
+                    // C(2a+1) weighs u(p + e_a), C(2a+2) weighs u(p - e_a)
+                    const Widen<3 * V> wp(&up[0][0]), wm(&um[0][0]);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
 #pragma unroll
                         for (int e = 0; e < V; ++e) {
-                            gv[1 + 2 * a][e] = __fma_rn(lam[e], (double)up[e], gv[1 + 2 * a][e]);
-                            gv[2 + 2 * a][e] = __fma_rn(lam[e], (double)um[e], gv[2 + 2 * a][e]);
+                            gv[1 + 2 * a][e] = __fma_rn(lam.d[e], wp.d[a * V + e], gv[1 + 2 * a][e]);
+                            gv[2 + 2 * a][e] = __fma_rn(lam.d[e], wm.d[a * V + e], gv[2 + 2 * a][e]);
                         }
-                    } else {
+                } else {
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int e = 0; e < V; ++e) up[a][e] = A::add(up[a][e], um[a][e]);
+                    const Widen<3 * V> w(&up[0][0]);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
                         const int m = 3 * (d - 1) + a + 1;
 #pragma unroll
-                        for (int e = 0; e < V; ++e) gv[m][e] = __fma_rn(lam[e], (double)A::add(up[e], um[e]), gv[m][e]);
+                        for (int e = 0; e < V; ++e) gv[m][e] = __fma_rn(lam.d[e], w.d[a * V + e], gv[m][e]);
                     }
                 }
             }
@@ -154,15 +202,24 @@ __global__ void __launch_bounds__(32 * BY) adjoint_grad_kernel(Layout L, AdjStep
     }
 }
 
+// Planes a thread walks in the kernels of this file, which keep nothing from one plane to the next:
+// as many as leave about 16 CTAs of 128 threads per SM (152), at most 16 (one plane after another
+// costs its full latency: 96 x 70 x 83, 16 planes a thread, took 188 us per gradient pass, 7-point,
+// and 36 us per transposed step). gridDim.z stays below its limit at any nz.
+static int adj_chunk(long long xy, int nz) {
+    long long c = xy * nz / (152 * 16);
+    c = c < 1 ? 1 : (c > 16 ? 16 : c);
+    const long long least = ((long long)nz + 65534) / 65535;
+    return (int)(c < least ? least : c);
+}
+
 template <int KIND, typename TF>
 static cudaError_t adj_grads(const Layout& L, const void* const* lam, const void* const* u, int n,
                              double* const* gC, cudaStream_t s) {
-    constexpr int BY = 4;
-    constexpr int V = 16 / sizeof(TF);
-    const int zchunk = 16;
-    dim3 block(32, BY, 1);
-    dim3 grid((unsigned)((L.nx + 32 * V - 1) / (32 * V)), (unsigned)((L.ny + BY - 1) / BY),
-              (unsigned)((L.nz + zchunk - 1) / zchunk));
+    constexpr int V = 16 / sizeof(TF), NT = 128;
+    dim3 grid((unsigned)(((long long)((L.nx + V - 1) / V) * L.ny + NT - 1) / NT), 1);
+    const int zchunk = adj_chunk(grid.x, L.nz);
+    grid.y = (unsigned)((L.nz + zchunk - 1) / zchunk);
     AdjGrad G{};
     for (int m = 0; m < KindTraits<KIND>::NC; ++m) G.g[m] = gC[m];
     for (int g0 = 0; g0 < n; g0 += ADJ_GROUP) {
@@ -172,7 +229,7 @@ static cudaError_t adj_grads(const Layout& L, const void* const* lam, const void
             S.lam[g] = static_cast<const TF*>(lam[g0 + g]);
             S.u[g] = static_cast<const TF*>(u[g0 + g]);
         }
-        adjoint_grad_kernel<KIND, TF, BY><<<grid, block, 0, s>>>(L, S, ng, G, zchunk);
+        adjoint_grad_kernel<KIND, TF, V, NT><<<grid, NT, 0, s>>>(L, S, ng, G, zchunk);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -213,10 +270,10 @@ static cudaError_t adj_step(const SweepArgs& a, const void* lam_in, void* lam_ou
     for (int m = 0; m < KindTraits<KIND>::NC; ++m) C.c[m] = static_cast<const TC*>(a.coef[m]);
     constexpr int BY = 4;
     constexpr int V = 16 / sizeof(TF);
-    const int zchunk = 16;
     dim3 block(32, BY, 1);
-    dim3 grid((unsigned)((L.nx + 32 * V - 1) / (32 * V)), (unsigned)((L.ny + BY - 1) / BY),
-              (unsigned)((L.nz + zchunk - 1) / zchunk));
+    dim3 grid((unsigned)((L.nx + 32 * V - 1) / (32 * V)), (unsigned)((L.ny + BY - 1) / BY), 1);
+    const int zchunk = adj_chunk((long long)grid.x * grid.y, L.nz);
+    grid.z = (unsigned)((L.nz + zchunk - 1) / zchunk);
     adjoint_vec_kernel<KIND, TF, TC, BY><<<grid, block, 0, s>>>(L, static_cast<const TF*>(lam_in),
                                                                 static_cast<TF*>(lam_out), C, zchunk);
     return cudaGetLastError();

@@ -252,3 +252,46 @@ def test_wavefront_backward_gives_the_plain_gradients(kind, shape, fdt, cdt, T, 
     tol = 1e-12 if fdt == "f64" else 2e-5
     rl, ru, rc = oracle.adjoint(kind, p.u0, p.coefs, target.double().cpu().numpy(), T)
     assert _rel(gu_w, ru) <= tol and _rel(gc_w, rc) <= tol
+
+
+@pytest.mark.parametrize("kind", ["7pt_var", "25pt_var"])
+def test_gradient_widening_of_every_class_of_value(kind):
+    """FP32 factors are widened to FP64 exactly whatever they are: one step's coefficient gradients
+    of a field with zeros, subnormals, huge values and infinities among ordinary ones are the FP64
+    products of the FP32 factors, bit for bit (NaN where the product is)."""
+    import torch
+    from paper_1410_5561_gb300.stencil import Stencil
+    nx, ny, nz = 37, 9, 8
+    s = Stencil(kind, nx, ny, nz)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    special = torch.tensor([0.0, -0.0, 1e-45, -1e-45, 1.1754943508222875e-38, 1e-39, 3.4e38, -3.4e38, float("inf"), 1.0],
+                           device="cuda")
+    u = torch.randn(nz, ny, nx, generator=g, device="cuda")
+    pick = torch.randint(0, 40, u.shape, generator=g, device="cuda")
+    u = torch.where(pick < 10, special[pick.clamp(max=9)], u)
+    lam = torch.randn(nz, ny, nx, generator=g, device="cuda")
+    pick = torch.randint(0, 40, u.shape, generator=g, device="cuda")
+    lam = torch.where(pick < 10, special[pick.clamp(max=9)], lam)
+    s.set_coeffs(arrays=[torch.zeros_like(u)] * s.ncoef)
+    s.set_field(u)
+    ws = s.adjoint_workspace(1)
+    s.run_checkpointed(1, 0, ws)
+    lp = s.new_field_array()
+    s.interior_of(lp).copy_(lam)
+    gu, gc = s.new_field_array(), [s.new_grad_array() for _ in range(s.ncoef)]
+    s.run_adjoint(1, 0, lp, gu, gc, ws)
+    r = s.layout.radius
+    p = torch.nn.functional.pad(u, (r,) * 6)
+
+    def at(axis, o):
+        i = [slice(r, n - r) for n in p.shape]
+        i[axis] = slice(r + o, p.shape[axis] - r + o)
+        return p[tuple(i)]
+    weights = [u]
+    for d in range(1, r + 1):
+        for axis in (2, 1, 0):
+            weights += [at(axis, d), at(axis, -d)] if kind == "7pt_var" else [at(axis, d) + at(axis, -d)]
+    for m in range(s.ncoef):
+        ref = 0.0 + lam.double() * weights[m].double()  # exact products: no rounding to compare
+        got = s.interior_of(gc[m])
+        assert torch.equal(got.nan_to_num(7.0, 8.0, 9.0), ref.nan_to_num(7.0, 8.0, 9.0)), m
