@@ -12,8 +12,10 @@
 //   memory one iteration before: one CTA barrier per iteration, whatever H.
 // * Input planes (and the planes of the coefficient arrays) arrive by tensor copies
 //   (cp.async.bulk.tensor) several iterations ahead, one thread issuing them; level 0's y
-//   neighbours are read from the copied plane. A coefficient plane stays in shared memory for
-//   the H iterations in which the levels pass it.
+//   neighbours are read from the copied plane. A thread reads its coefficient vectors from the
+//   copied plane once and keeps them in registers for the H iterations in which the levels pass
+//   it: read again by every level they took most of the shared-memory bandwidth (384^3 FP32 300 ->
+//   425 GLUP/s, BF16, kept as stored and widened at each use, 363 -> 484).
 // * Tiles overlap: a level's outermost columns / rows are wrong where the tile ends inside the
 //   domain, one more per level, so neighbouring tiles recompute 4 columns (one vector) and
 //   H - 1 rows on each side, and chunks of z recompute H planes. CTAs of a launch never wait
@@ -29,6 +31,8 @@
 // blocked_impl.cuh 24; HBM at 3 bytes per update is the next bound (about 2100 GLUP/s). Measured,
 // 7-point constant, GLUP/s, AUTO before (diamonds) -> this: 1024^3 856 -> 1898, 512^3 727 -> 1610,
 // 256^3 394 -> 1037, 301 x 257 x 199 241 -> 861, 64^3 16 -> 64 (plain sweep: 702, 678, 511, 473, 28).
+// 7-point variable 384^3: FP32 200 -> 425 (HBM at 5.2 TB/s, 13 bytes per update), BF16 253 -> 484
+// (issue and latency of the widening).
 #pragma once
 #include <limits.h>
 
@@ -63,15 +67,19 @@ __device__ __forceinline__ void ov_sts(uint32_t a, const V4& x) {
 __device__ __forceinline__ void ov_stg(float* p, const V4& x) {
     *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(x.a.r, x.b.r);
 }
-// One thread's coefficient vector, widened to FP32.
+// One thread's coefficient vector as it is stored, and widened to FP32.
 template <typename TC> struct OvCoef;
 template <> struct OvCoef<float> {
-    static __device__ __forceinline__ V4 ld(uint32_t a, uint32_t tok) { return ov_lds(a, tok); }
+    V4 v;
+    __device__ __forceinline__ void ld(uint32_t a, uint32_t tok) { v = ov_lds(a, tok); }
+    __device__ __forceinline__ V4 get() const { return v; }
 };
 template <> struct OvCoef<__nv_bfloat16> {
-    static __device__ __forceinline__ V4 ld(uint32_t a, uint32_t tok) {
-        uint32_t u0, u1;
+    uint32_t u0, u1;
+    __device__ __forceinline__ void ld(uint32_t a, uint32_t tok) {
         asm("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(u0), "=r"(u1) : "r"(a), "r"(tok));
+    }
+    __device__ __forceinline__ V4 get() const {
         // exact: a BF16 value is the upper half of its FP32 value
         return V4{F2::pack(__uint_as_float(u0 << 16), __uint_as_float(u0 & 0xffff0000u)),
                   F2::pack(__uint_as_float(u1 << 16), __uint_as_float(u1 & 0xffff0000u))};
@@ -110,8 +118,8 @@ struct OvCtl {
     int stall_item;
 };
 
-// Sizes of one instantiation. PD: field planes copied ahead; CR: coefficient planes held (the
-// H that the levels use and those in flight).
+// Sizes of one instantiation. PD: field planes copied ahead; CR: coefficient planes held (the one
+// being read and those in flight).
 template <int KIND, typename TC, int NW, int RB, int H, int PD, int CR>
 struct OvCfg {
     static constexpr int NC = KindTraits<KIND>::NC;
@@ -125,13 +133,13 @@ struct OvCfg {
     // 16-byte boundary, and the tiles' first columns are odd multiples of 4 elements in the arrays
     static constexpr int CX0 = sizeof(TC) == 2 ? 4 : 0, CXW = OV_X + 2 * CX0;
     static constexpr int CROWB = CXW * (int)sizeof(TC);
-    static constexpr int CARRB = YT * CROWB;               // one coefficient array's plane
-    static constexpr int CPLANEB = NC * CARRB;
+    static constexpr int CARRB = (YT * CROWB + 127) / 128 * 128;  // one coefficient array's plane
+    static constexpr int CPLANEB = NC * CARRB, CTXB = NC * YT * CROWB;
     static constexpr int COEF0 = RING * PLANEB;
     static constexpr int PUB0 = COEF0 + (NC > 0 ? CR * CPLANEB : 0);
     static constexpr int BAR0 = PUB0 + 2 * (H - 1) * PUBL;
     static constexpr int BYTES = BAR0 + (RING + CR) * 8;
-    static_assert(PLANEB % 128 == 0 && CARRB % 128 == 0, "box destinations stay 128-byte aligned");
+    static_assert(PLANEB % 128 == 0 && PUB0 % 16 == 0, "box destinations stay 128-byte aligned");
 };
 
 // The copy rings' positions, carried from one tile to the next in shared memory: slot and phase of
@@ -177,7 +185,7 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
     };
     auto ccopy = [&](int z, int slot) {
         if constexpr (NC > 0) {
-            mbar_arrive_expect_tx(cbar + 8 * slot, S::CPLANEB);
+            mbar_arrive_expect_tx(cbar + 8 * slot, S::CTXB);
 #pragma unroll
             for (int m = 0; m < NC; ++m)
                 tma_load_3d(s0 + S::COEF0 + slot * S::CPLANEB + m * S::CARRB, &A.cmap[m], L.xo + xl - S::CX0, yl + 1,
@@ -228,6 +236,7 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
 #pragma unroll
             for (int i = 0; i < RB; ++i) win[l][r][i] = hvv;
 
+    OvCoef<TC> co[NC > 0 ? 3 : 1][NC > 0 ? NC : 1][RB];  // planes s - 1, s - 2, s - 3, rotating as the windows
     int sl = r0.fs, slf = (r0.fs + PD) % S::RING;      // ring slots of field planes s and s + PD
     uint32_t so = (uint32_t)(sl * S::PLANEB);          // byte offsets of field planes s and s - 1
     uint32_t sc = (uint32_t)((sl == 0 ? S::RING - 1 : sl - 1) * S::PLANEB);
@@ -253,10 +262,10 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
         if (threadIdx.x == 0 && lost == INT_MAX) {
             if (s + PD < zl) copy(s + PD, slf);
             if (NC > 0) {
-                // the slot of plane s - 1 - HL, which the last level has left: plane s - 1 + CR - HL
-                // (those up to cb + CR - 2 were copied at the start)
-                const int z = s - 1 + CR - HL;
-                if (z >= cb + CR - 1 && z < ce) ccopy(z, cl >= HL ? cl - HL : cl - HL + CR);
+                // the slot of plane s - 2, read in the iteration before: plane s - 2 + CR (those up to
+                // cb + CR - 2 were copied at the start)
+                const int z = s - 2 + CR;
+                if (z >= cb + CR - 1 && z < ce) ccopy(z, cl >= 1 ? cl - 1 : CR - 1);
             }
         }
         if (STEADY || s < zl) arrived(bar + 8 * sl, ph, s);
@@ -266,6 +275,14 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
             if (STEADY || s < zl) {
 #pragma unroll
                 for (int i = 0; i < RB; ++i) win[0][ZP][i] = ov_lds(own + so + (uint32_t)(i * S::ROWB), tw);
+            }
+            if constexpr (NC > 0) {
+                // (a plane that was not copied feeds only points whose results are not used)
+                const uint32_t cq = cown + (uint32_t)(cl * S::CPLANEB);
+#pragma unroll
+                for (int i = 0; i < RB; ++i)
+#pragma unroll
+                    for (int m = 0; m < NC; ++m) co[PH % 3][m][i].ld(cq + (uint32_t)(m * S::CARRB + i * S::CROWB), tw);
             }
             const uint32_t prd = pub + (par ^ (uint32_t)((H - 1) * S::PUBL));
             const uint32_t pwr = pub + par;
@@ -283,8 +300,6 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
                     up = ov_lds(q + (PR - 1) * S::ROWB, tok);  // last row of the warp above
                     dn = ov_lds(q + 2 * PR * S::ROWB, tok);    // first row of the warp below
                 }
-                const uint32_t cq = cown + (uint32_t)((cl >= l ? cl - l : cl - l + CR) * S::CPLANEB);
-                (void)cq;
 #pragma unroll
                 for (int i = 0; i < RB; ++i) {
                     const V4 c = win[l][ZC][i];
@@ -308,13 +323,13 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
                     } else {
                         // Listing 2's order; the x terms point by point (the neighbours are
                         // not register pairs), the others as packed pairs
-                        const uint32_t ca = cq + (uint32_t)(i * S::CROWB);
-                        V4 k = OvCoef<TC>::ld(ca, tw);
-                        V4 r{F2::mul(k.a, c.a), F2::mul(k.b, c.b)};
+                        const auto& k = co[NC > 0 ? (PH + 3 - l % 3) % 3 : 0];
+                        V4 q = k[0][i].get();
+                        V4 r{F2::mul(q.a, c.a), F2::mul(q.b, c.b)};
                         float o[4], kp[4], km[4];
                         r.get(o);
-                        OvCoef<TC>::ld(ca + S::CARRB, tw).get(kp);
-                        OvCoef<TC>::ld(ca + 2 * S::CARRB, tw).get(km);
+                        k[NC > 0 ? 1 : 0][i].get().get(kp);
+                        k[NC > 0 ? 2 : 0][i].get().get(km);
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             o[e] = Ar<float>::fma(kp[e], e < 3 ? v[e < 3 ? e + 1 : 0] : xp3, o[e]);
@@ -322,9 +337,9 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
                         }
                         r = V4::of(o);
                         auto term = [&](int m, const V4& u) {
-                            k = OvCoef<TC>::ld(ca + (uint32_t)(m * S::CARRB), tw);
-                            r.a = F2::fma(k.a, u.a, r.a);
-                            r.b = F2::fma(k.b, u.b, r.b);
+                            q = k[NC > 0 ? m : 0][i].get();
+                            r.a = F2::fma(q.a, u.a, r.a);
+                            r.b = F2::fma(q.b, u.b, r.b);
                         };
                         term(3, yp);
                         term(4, ym);
@@ -332,7 +347,7 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
                         term(6, zm);
                         out[i] = r;
                     }
-                                            if constexpr (EDGE == 2 || !STEADY) {
+                    if constexpr (EDGE == 2 || !STEADY) {
                         float o[4];
                         out[i].get(o);
 #pragma unroll
@@ -406,7 +421,7 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
     else walk(std::integral_constant<int, 0>{});
     if (threadIdx.x == 0 && lost != INT_MAX) {
         // the copies still in flight end before the CTA goes on (bounded): the last one of every slot
-        const int fl = min(zl, lost + PD + 1) - 1 - s_begin, cf = min(ce, max(cb + CR - 1, lost + CR - HL)) - 1 - cb;
+        const int fl = min(zl, lost + PD + 1) - 1 - s_begin, cf = min(ce, max(cb + CR - 1, lost + CR - 1)) - 1 - cb;
         for (int p = max(0, fl - S::RING + 1); p <= fl; ++p)
             mbar_wait(bar + 8 * ((r0.fs + p) % S::RING), (uint32_t)(r0.fp ^ ((r0.fs + p) / S::RING & 1)), status);
         for (int p = max(0, cf - CR + 1); NC > 0 && p <= cf; ++p)
