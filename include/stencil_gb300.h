@@ -276,16 +276,19 @@ int stencil_copy(void* dst, const void* src, size_t bytes, int ctas, void* cuda_
 int stencil_probe_fma(int dtype, int iters, void* scratch, void* cuda_stream, double* seconds, double* flops);
 
 /* ---- Batch: many independent grids advanced by one persistent launch.
- * Every grid runs the blocked schedule (Section II-A) with one tile covering
- * its whole x extent; tiles of all grids sit in one dependency-ordered list
- * and the CTAs of one persistent kernel pop them from an atomic counter, each
- * waiting (with a bounded spin) until the diamonds below it have published
- * their results: the GPU form of the paper's queue of ready diamond tiles. */
+ * The tiles of all grids sit in one dependency-ordered list and the CTAs of one
+ * persistent kernel pop them from an atomic counter, each waiting (with a
+ * bounded spin) until the tiles it depends on have published their results: the
+ * GPU form of the paper's queue of ready diamond tiles. Grids of the 7-point
+ * stencils with an FP32 field run overlapped tiles (as STENCIL_OVERLAP), the
+ * list following the grids' chains of passes; the others run the blocked
+ * schedule (Section II-A) with one tile covering a grid's whole x extent. */
 typedef struct stencil_batch* stencil_batch_t; /* opaque, owned by the library */
 
 /* Plan a batch: grids[q] (bound, same kind and dtypes) advances by T[q] >= 0 steps
- * per launch. tuning: dw, nf (1 or 2) and warps are used for every grid; xtile is
- * ignored. STENCIL_EINVAL if a grid cannot use the tuning. */
+ * per launch. tuning: dw, nf (1 or 2) and warps are used for every grid that runs the
+ * blocked schedule; xtile is ignored. STENCIL_EINVAL if a grid cannot use the tuning,
+ * whichever schedule it runs. */
 int stencil_batch_create(stencil_batch_t* out, const stencil_t* grids, const int* T, int n,
                          const stencil_tuning* tuning);
 

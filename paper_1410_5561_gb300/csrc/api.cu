@@ -746,8 +746,7 @@ int stencil_batch_set_wait_limit(stencil_batch_t b, unsigned spins) {
 int stencil_batch_inject_stall(stencil_batch_t b, int item) {
     if (!b || item < 0 || item >= b->bl.nitems) return STENCIL_EINVAL;
     if (!b->bound) return STENCIL_EUNBOUND;
-    b->bl.items[item].dep[2] = b->bl.nitems;  // the extra completion flag, which no tile ever sets
-    if (batch_reupload_items(&b->bl, b->stream) != cudaSuccess) return STENCIL_ECUDA;
+    if (batch_stall(&b->bl, item, b->stream) != cudaSuccess) return STENCIL_ECUDA;
     return STENCIL_OK;
 }
 

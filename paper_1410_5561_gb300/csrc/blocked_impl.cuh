@@ -1397,7 +1397,7 @@ static int batch_items(const BatchGrid* g, int n, int dw, std::vector<BatchItem>
 }
 
 #ifdef STG_BLOCKED_MAIN
-cudaError_t batch_plan(const BatchGrid* g, int n, const BlockedTune& tn, BatchLaunch* bl) {
+cudaError_t batch_plan(const BatchGrid* g, int n, const BlockedTune& tn, BatchLaunch* bl, size_t limit) {
     if (n < 1) return cudaErrorInvalidValue;
     const SweepArgs& a0 = g[0].a;
     int K = 1;
@@ -1441,10 +1441,11 @@ cudaError_t batch_plan(const BatchGrid* g, int n, const BlockedTune& tn, BatchLa
     bl->off_counters = off;  // head, status, gdone[n], done[nitems + 1] (the extra flag is never set)
     bl->counter_bytes = sizeof(int) * (size_t)(2 + n + nitems + 1);
     off += align256(bl->counter_bytes);
-    bl->bytes = off;
+    bl->bytes = bl->diamond_bytes = off;
     bl->items = items;
     bl->ntiles = ntiles;
-    return cudaSuccess;
+    // the 7-point stencils in FP32: overlapped tiles, faster on every batch measured
+    return overlap_batch_plan(g, n, limit, bl);
 }
 #endif  // STG_BLOCKED_MAIN
 
@@ -1479,6 +1480,7 @@ cudaError_t batch_upload(const BatchGrid* g, int n, const BlockedTune& tn, Batch
                          cudaStream_t s) {
     char* w = static_cast<char*>(ws);
     bl->ws = w;
+    if (bl->overlap) return overlap_batch_upload(g, n, bl, w, s);
     if (bl->fdt == DT_F64) return batch_upload_t<double, double>(g, n, tn, bl, w, s);
     if (bl->cdt == DT_BF16) return batch_upload_t<float, __nv_bfloat16>(g, n, tn, bl, w, s);
     return batch_upload_t<float, float>(g, n, tn, bl, w, s);
@@ -1486,9 +1488,18 @@ cudaError_t batch_upload(const BatchGrid* g, int n, const BlockedTune& tn, Batch
 #endif  // STG_BLOCKED_MAIN
 
 #ifdef STG_BLOCKED_MAIN
-cudaError_t batch_reupload_items(BatchLaunch* bl, cudaStream_t s) {
-    cudaError_t e = cudaMemcpyAsync(bl->ws + bl->off_items, bl->items.data(), sizeof(BatchItem) * bl->items.size(),
-                                    cudaMemcpyHostToDevice, s);
+cudaError_t batch_stall(BatchLaunch* bl, int item, cudaStream_t s) {
+    cudaError_t e;
+    if (bl->overlap) {
+        OvItem& it = bl->ov_items[item];
+        if (it.g >= 0) it.g = ~it.g;
+        e = cudaMemcpyAsync(bl->ws + bl->off_items, bl->ov_items.data(), sizeof(OvItem) * bl->ov_items.size(),
+                            cudaMemcpyHostToDevice, s);
+    } else {
+        bl->items[item].dep[2] = bl->nitems;  // the extra completion flag, which no tile ever sets
+        e = cudaMemcpyAsync(bl->ws + bl->off_items, bl->items.data(), sizeof(BatchItem) * bl->items.size(),
+                            cudaMemcpyHostToDevice, s);
+    }
     if (e) return e;
     return cudaStreamSynchronize(s);
 }
@@ -1537,6 +1548,7 @@ cudaError_t batch_launch_t(const BatchLaunch& bl, cudaStream_t s) {
 
 #ifdef STG_BLOCKED_MAIN
 cudaError_t batch_launch(const BatchLaunch& bl, cudaStream_t s) {
+    if (bl.overlap) return overlap_batch_launch(bl, s);
     switch (bl.kind) {
         case K7C:
             if (bl.fdt == DT_F32) return batch_launch_t<K7C, float, float>(bl, s);

@@ -143,9 +143,19 @@ struct BatchGrid {
     int T;       // steps to advance
 };
 
+// Item of an overlapped-tile batch: tile t of pass p of grid g (~g: the stall hook's item).
+struct OvItem {
+    int g, p, t;
+};
+
 struct BatchLaunch {
     int kind, fdt, cdt, K, nf, threads, ngrids, nitems;
     size_t smem, bytes, counter_bytes;
+    size_t diamond_bytes;  // workspace of the diamond schedule (bytes covers either schedule)
+    bool overlap = false;  // overlapped tiles instead of diamonds (overlap.cu)
+    std::vector<OvItem> ov_items;
+    std::vector<int> ov_zc, ov_first;  // per grid: planes per chunk, first completion counter
+    size_t off_first = 0, off_flip = 0;
     size_t off_grids, off_items, off_ntiles, off_parity, off_counters;
     unsigned spin_limit = 1u << 24;
     char* ws = nullptr;
@@ -153,10 +163,18 @@ struct BatchLaunch {
     std::vector<int> ntiles;
 };
 
-cudaError_t batch_plan(const BatchGrid* g, int n, const BlockedTune& tn, BatchLaunch* bl);
+// limit: most workspace bytes the overlapped-tile form may take (the diamonds' size does not depend on it).
+cudaError_t batch_plan(const BatchGrid* g, int n, const BlockedTune& tn, BatchLaunch* bl, size_t limit = (size_t)-1);
 cudaError_t batch_upload(const BatchGrid* g, int n, const BlockedTune& tn, BatchLaunch* bl, void* ws, cudaStream_t s);
-cudaError_t batch_reupload_items(BatchLaunch* bl, cudaStream_t s);
+// Makes item `item` of the uploaded plan wait on a flag that nothing sets (test hook).
+cudaError_t batch_stall(BatchLaunch* bl, int item, cudaStream_t s);
 cudaError_t batch_launch(const BatchLaunch& bl, cudaStream_t s);
+
+// The overlapped-tile form of a batch whose grids all allow it: the plan (bl->overlap stays false
+// where the form does not apply or its workspace would exceed limit bytes), the upload, the launch.
+cudaError_t overlap_batch_plan(const BatchGrid* g, int n, size_t limit, BatchLaunch* bl);
+cudaError_t overlap_batch_upload(const BatchGrid* g, int n, BatchLaunch* bl, char* ws, cudaStream_t s);
+cudaError_t overlap_batch_launch(const BatchLaunch& bl, cudaStream_t s);
 
 // Read access to a bound grid handle for batch planning (STENCIL_EUNBOUND if unbound),
 // and the parity update after a batch launch.

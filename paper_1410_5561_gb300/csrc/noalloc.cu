@@ -69,8 +69,8 @@ extern "C" int stencil_batch_run_noalloc(const stencil_t* grids, const int* T, i
         if (!on_device(g[q].field[0], dev) || !on_device(g[q].field[1], dev)) return STENCIL_EINVAL;
     BlockedTune tn{tuning->dw, tuning->nf, tuning->warps, 0};
     BatchLaunch bl;
-    if (batch_plan(g.data(), n, tn, &bl) != cudaSuccess) return STENCIL_EINVAL;
-    if (bl.bytes > NOALLOC_SCRATCH_BYTES) return STENCIL_EINVAL;  // plan larger than the static scratch
+    if (batch_plan(g.data(), n, tn, &bl, NOALLOC_SCRATCH_BYTES) != cudaSuccess) return STENCIL_EINVAL;
+    if (bl.diamond_bytes > NOALLOC_SCRATCH_BYTES) return STENCIL_EINVAL;  // plan larger than the static scratch
     void* ws = nullptr;
     if (scratch_address(&ws) != cudaSuccess) return STENCIL_ECUDA;
     if (batch_upload(g.data(), n, tn, &bl, ws, s) != cudaSuccess) return STENCIL_ECUDA;

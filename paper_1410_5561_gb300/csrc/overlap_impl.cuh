@@ -153,24 +153,27 @@ __device__ __forceinline__ int ov_uniform(int v) { return __shfl_sync(0xffffffff
 
 // One tile of one pass, the whole CTA. HL: the levels it computes (H, or 1 in a short pass; the
 // geometry is that of H either way). Thread 0 issues the copies.
-template <int KIND, typename TC, int NW, int RB, int H, int PD, int CR, int HL>
+// In a batch the grid's constants come from global memory: broadcast, so that they are uniform too.
+template <int KIND, typename TC, int NW, int RB, int H, int PD, int CR, int HL, bool BATCH>
 __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, const int bx, const int by, const int bz,
                                              const uint32_t s0, OvRings* ring, int* status) {
     using S = OvCfg<KIND, TC, NW, RB, H, PD, CR>;
     constexpr int YT = S::YT, YH = S::YH, NC = S::NC, PR = S::PR;
     const int lane = threadIdx.x & 31, w = ov_uniform((int)threadIdx.x >> 5);
-    const Layout& L = A.L;
-    const int nx = L.nx, ny = L.ny, nz = L.nz;
+    auto uni = [](int v) { return BATCH ? ov_uniform(v) : v; };
+    const int nx = uni(A.L.nx), ny = uni(A.L.ny), nz = uni(A.L.nz), px = uni(A.L.px), py = uni(A.L.py), xo = uni(A.L.xo);
+    const int ntx = uni(A.ntx), nty = uni(A.nty), zc = uni(A.zc);
+    const float c0 = __int_as_float(uni(__float_as_int(A.c0))), c1 = __int_as_float(uni(__float_as_int(A.c1)));
     const int xs = ov_first(bx, OV_X, OV_V), ys = ov_first(by, YT, YH);  // first owned column and row
-    const int xe = bx == A.ntx - 1 ? nx : ov_first(bx + 1, OV_X, OV_V);
-    const int ye = by == A.nty - 1 ? ny : ov_first(by + 1, YT, YH);
+    const int xe = bx == ntx - 1 ? nx : ov_first(bx + 1, OV_X, OV_V);
+    const int ye = by == nty - 1 ? ny : ov_first(by + 1, YT, YH);
     // the tile's first column and row; the last tile of several starts up to RB - 1 rows earlier,
     // so that the domain ends with a warp's last row
     const int xl = bx == 0 ? 0 : xs - OV_V;
-    const int yl = by == 0 ? 0 : (by == A.nty - 1 ? ny - (ny - (ys - YH) + RB - 1) / RB * RB : ys - YH);
+    const int yl = by == 0 ? 0 : (by == nty - 1 ? ny - (ny - (ys - YH) + RB - 1) / RB * RB : ys - YH);
     const int x = xl + 4 * lane, y0 = yl + w * RB;  // this thread's first column and row
-    const int z0 = bz * A.zc, z1 = min(nz, z0 + A.zc);
-    const float hv = A.hv;
+    const int z0 = bz * zc, z1 = min(nz, z0 + zc);
+    const float hv = __int_as_float(uni(__float_as_int(A.hv)));
     const V4 hvv{F2::pack(hv, hv), F2::pack(hv, hv)};
 
     const bool live = y0 < ny;  // warp-uniform
@@ -181,14 +184,14 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
     const uint32_t bar = s0 + S::BAR0, cbar = bar + 8 * S::RING;
     auto copy = [&](int z, int slot) {
         mbar_arrive_expect_tx(bar + 8 * slot, S::PLANEB);
-        tma_load_3d(s0 + slot * S::PLANEB, &A.map[src], L.xo + xl, yl, z + 1, bar + 8 * slot);
+        tma_load_3d(s0 + slot * S::PLANEB, &A.map[src], xo + xl, yl, z + 1, bar + 8 * slot);
     };
     auto ccopy = [&](int z, int slot) {
         if constexpr (NC > 0) {
             mbar_arrive_expect_tx(cbar + 8 * slot, S::CTXB);
 #pragma unroll
             for (int m = 0; m < NC; ++m)
-                tma_load_3d(s0 + S::COEF0 + slot * S::CPLANEB + m * S::CARRB, &A.cmap[m], L.xo + xl - S::CX0, yl + 1,
+                tma_load_3d(s0 + S::COEF0 + slot * S::CPLANEB + m * S::CARRB, &A.cmap[m], xo + xl - S::CX0, yl + 1,
                             z + 1, cbar + 8 * slot);
         }
     };
@@ -215,9 +218,9 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
         }
     }
 
-    const size_t plane = L.plane();
+    const size_t plane = (size_t)px * py;
     const bool xown = x >= xs && x < xe;
-    float* dp = A.f[src ^ 1] + L.at(xown ? x : 0, live ? y0 : 0, 0);
+    float* dp = A.f[src ^ 1] + plane + (size_t)((live ? y0 : 0) + 1) * px + (xo + (xown ? x : 0));  // row y0, z = 0
     const bool xfull = x + 4 <= nx;
     bool st[RB];
 #pragma unroll
@@ -315,7 +318,10 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
                         xp3 = redge ? hv : xp3;
                     }
                     if constexpr (KIND == K7C) {
-                        const F2 c0p = F2::pack(A.c0, A.c0), c1p = F2::pack(A.c1, A.c1);
+                        // (one grid: read where they are used, from the parameter bank: 1905 GLUP/s at
+                        // 1024^3, 1780 with both held in registers)
+                        const float q0 = BATCH ? c0 : A.c0, q1 = BATCH ? c1 : A.c1;
+                        const F2 c0p = F2::pack(q0, q0), c1p = F2::pack(q1, q1);
                         const F2 sxa = F2::pack(Ar<float>::add(v[1], xm0), Ar<float>::add(v[2], v[0]));
                         const F2 sxb = F2::pack(Ar<float>::add(v[3], v[1]), Ar<float>::add(xp3, v[2]));
                         out[i].a = upd7c_x2(c0p, c1p, c.a, sxa, yp.a, ym.a, zp.a, zm.a);
@@ -367,13 +373,13 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
 #pragma unroll
                     for (int i = 0; i < RB; ++i) {
                         if (EDGE < 2 || xfull) {
-                            if (st[i]) ov_stg(d + (size_t)i * L.px, out[i]);
+                            if (st[i]) ov_stg(d + (size_t)i * px, out[i]);
                         } else if (st[i]) {
                             float o[4];
                             out[i].get(o);
 #pragma unroll
                             for (int e = 0; e < 4; ++e)
-                                if (x + e < nx) d[(size_t)i * L.px + e] = o[e];
+                                if (x + e < nx) d[(size_t)i * px + e] = o[e];
                         }
                     }
                 }
@@ -504,14 +510,128 @@ __global__ void __launch_bounds__(NW * 32, 1) overlap_kernel(const __grid_consta
         if (i >= items) break;
         const int p = i / tiles, t = i - p * tiles;
         const int bx = t % G.ntx, by = t / G.ntx % G.nty, bz = t / (G.ntx * G.nty), src = (G.p0 + p) & 1;
-        if (p < G.full) overlap_tile<KIND, TC, NW, RB, H, PD, CR, H>(G, src, bx, by, bz, s0, &s_ring, C.status);
-        else overlap_tile<KIND, TC, NW, RB, H, PD, CR, 1>(G, src, bx, by, bz, s0, &s_ring, C.status);
+        if (p < G.full) overlap_tile<KIND, TC, NW, RB, H, PD, CR, H, false>(G, src, bx, by, bz, s0, &s_ring, C.status);
+        else overlap_tile<KIND, TC, NW, RB, H, PD, CR, 1, false>(G, src, bx, by, bz, s0, &s_ring, C.status);
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();  // with the barrier before it: the CTA's stores are visible GPU-wide
             ov_st_release(C.done + t, p + 1);
         }
     }
+}
+
+// The same over the items of many grids, in the order that the host planned (every item after those
+// it waits for). Each grid's parity is read from and, once its last tile has finished, written to
+// device memory, so that the launch can be replayed.
+struct OvBatchArgs {
+    const OvGrid* grids;
+    const OvItem* items;
+    int nitems;
+    int* head;
+    int* status;        // 1: a wait gave up
+    int* never;
+    int* gdone;         // per grid: items finished in this launch
+    int* done;          // per tile (grid q from first[q]): passes finished
+    const int* first;
+    const int* ntiles;  // per grid: items per launch
+    const int* parity_flip;  // per grid: T & 1
+    int* parity;
+    unsigned spin_limit;
+};
+
+template <int KIND, typename TC, int NW, int RB, int H, int PD, int CR>
+__global__ void __launch_bounds__(NW * 32, 1) overlap_batch_kernel(const OvBatchArgs B) {
+    using S = OvCfg<KIND, TC, NW, RB, H, PD, CR>;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ int s_item, s_src;
+    __shared__ OvRings s_ring;
+    const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    if (threadIdx.x == 0) {
+        for (int p = 0; p < S::RING + CR; ++p) mbar_init(s0 + S::BAR0 + 8 * p, 1);
+        mbar_init_fence();
+        s_ring = OvRings{0, 0, 0, 0};
+    }
+    const OvCtl C{B.status, B.never, B.head, B.done, B.spin_limit, -1};
+    int next = 0;  // thread 0: the item to do next
+    if (threadIdx.x == 0) next = atomicAdd(B.head, 1);
+    for (;;) {
+        if (threadIdx.x < 32) {
+            const int i = __shfl_sync(0xffffffffu, next, 0);
+            if (i < B.nitems) {
+                const OvItem it = B.items[i];
+                const bool stall = it.g < 0;
+                const int g = stall ? ~it.g : it.g;
+                const OvGrid& G = B.grids[g];
+                const int ntx = G.ntx, nty = G.nty;
+                if (it.p > 0)
+                    ov_wait_tiles(C, B.done + B.first[g], ntx, nty, G.ntz, it.t % ntx, it.t / ntx % nty, it.t / (ntx * nty),
+                                  it.p);
+                if (threadIdx.x == 0) {
+                    if (stall) ov_wait_flag(C, B.never, 1);
+                    next = atomicAdd(B.head, 1);
+                    const int p0 = *(volatile int*)(B.parity + g);
+                    s_src = (p0 + it.p) & 1;
+                    // what other CTAs stored (acquired above), and the grid's maps (written by the
+                    // upload), are read through the copy engine next
+                    fence_proxy_async_global();
+                    tma_map_acquire(&G.map[s_src]);
+                    for (int m = 0; m < S::NC; ++m) tma_map_acquire(&G.cmap[m]);
+                }
+            }
+            if (threadIdx.x == 0) s_item = i;
+        }
+        __syncthreads();
+        const int i = ov_uniform(s_item);
+        if (i >= B.nitems) break;
+        const int src = ov_uniform(s_src);
+        const int ig = ov_uniform(B.items[i].g), g = ig < 0 ? ~ig : ig;
+        const int p = ov_uniform(B.items[i].p), t = ov_uniform(B.items[i].t);
+        const OvGrid& G = B.grids[g];
+        const int ntx = ov_uniform(G.ntx), nty = ov_uniform(G.nty);
+        const int bx = t % ntx, by = t / ntx % nty, bz = t / (ntx * nty);
+        if (p < ov_uniform(G.full)) overlap_tile<KIND, TC, NW, RB, H, PD, CR, H, true>(G, src, bx, by, bz, s0, &s_ring, C.status);
+        else overlap_tile<KIND, TC, NW, RB, H, PD, CR, 1, true>(G, src, bx, by, bz, s0, &s_ring, C.status);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();  // with the barrier before it: the CTA's stores are visible GPU-wide
+            ov_st_release(B.done + B.first[g] + t, p + 1);
+            // the last item of the grid: every other one has read the parity
+            if (atomicAdd(B.gdone + g, 1) == B.ntiles[g] - 1) B.parity[g] ^= B.parity_flip[g];
+        }
+    }
+}
+
+// Host-side description of one grid (everything but the z chunk and the pass counts).
+template <int KIND, typename TC, int NW, int RB, int H, int PD, int CR>
+cudaError_t overlap_grid(const SweepArgs& a, void* const field[2], OvGrid* G) {
+    using S = OvCfg<KIND, TC, NW, RB, H, PD, CR>;
+    const Layout& L = a.L;
+    for (int i = 0; i < 2; ++i) {
+        if (!tma_encode_3d(&G->map[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, field[i], L, OV_X, S::YT + 2))
+            return cudaErrorNotSupported;
+        G->f[i] = static_cast<float*>(field[i]);
+    }
+    for (int m = 0; m < S::NC; ++m)
+        if (!tma_encode_3d(&G->cmap[m], sizeof(TC) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                           (int)sizeof(TC), a.coef[m], L, S::CXW, S::YT))
+            return cudaErrorNotSupported;
+    G->L = L;
+    G->c0 = (float)a.c0;
+    G->c1 = (float)a.c1;
+    G->hv = (float)a.halo;
+    G->ntx = ov_tiles(L.nx, OV_X, OV_V);
+    G->nty = ov_tiles(L.ny, S::YT, S::YH);
+    return cudaSuccess;
+}
+
+template <int KIND, typename TC, int NW, int RB, int H, int PD, int CR>
+cudaError_t overlap_batch_go(const OvBatchArgs& B, int sms, cudaStream_t st) {
+    using S = OvCfg<KIND, TC, NW, RB, H, PD, CR>;
+    auto kfn = overlap_batch_kernel<KIND, TC, NW, RB, H, PD, CR>;
+    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES);
+    if (e) return e;
+    kfn<<<(unsigned)(B.nitems < sms ? B.nitems : sms), NW * 32, S::BYTES, st>>>(B);
+    return cudaGetLastError();
 }
 
 // T steps in one launch: T / H passes of H steps and T % H of one. With an odd H every pass flips
@@ -529,21 +649,7 @@ cudaError_t overlap_launch(const SweepArgs& a, void* const field[2], int p0, int
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
     if ((e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES))) return e;
     OvGrid G{};
-    for (int i = 0; i < 2; ++i) {
-        if (!tma_encode_3d(&G.map[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, field[i], L, OV_X, S::YT + 2))
-            return cudaErrorNotSupported;
-        G.f[i] = static_cast<float*>(field[i]);
-    }
-    for (int m = 0; m < S::NC; ++m)
-        if (!tma_encode_3d(&G.cmap[m], sizeof(TC) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-                           (int)sizeof(TC), a.coef[m], L, S::CXW, S::YT))
-            return cudaErrorNotSupported;
-    G.L = L;
-    G.c0 = (float)a.c0;
-    G.c1 = (float)a.c1;
-    G.hv = (float)a.halo;
-    G.ntx = ov_tiles(L.nx, OV_X, OV_V);
-    G.nty = ov_tiles(L.ny, S::YT, S::YH);
+    if ((e = overlap_grid<KIND, TC, NW, RB, H, PD, CR>(a, field, &G))) return e;
     const long long columns = (long long)G.ntx * G.nty;
     G.zc = ov_chunk(columns, L.nz, H, sms, chunks);
     G.ntz = (L.nz + G.zc - 1) / G.zc;

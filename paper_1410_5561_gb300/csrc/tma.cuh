@@ -59,6 +59,12 @@ __device__ __forceinline__ void fence_proxy_async_global() {
     asm volatile("fence.proxy.async.global;\n" ::: "memory");
 }
 
+// Makes a tensor map in global memory, written before the launch, visible to this CTA's copies (a
+// cached copy of what the same address held earlier is dropped).
+__device__ __forceinline__ void tma_map_acquire(const CUtensorMap* map) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 // One box of a 3D tensor map at element coordinates (x, y, z) into shared memory.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t mbar) {
     asm volatile(
