@@ -13,6 +13,7 @@
 // condition of the transpose automatic. Coefficient gradients accumulate in FP64.
 #include "adjoint_column.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace stg {
 
@@ -27,6 +28,7 @@ template <int KIND, typename TF, typename TC, int BY>
 __global__ void __launch_bounds__(32 * BY) adjoint_vec_kernel(Layout L, const TF* __restrict__ lam_in,
                                                               TF* __restrict__ lam_out, CoefPtrs<TC> C, int zchunk) {
     constexpr int V = 16 / sizeof(TF);
+    dependent_begin();
     const int i0 = (blockIdx.x * 32 + threadIdx.x) * V;
     const int j = blockIdx.y * BY + threadIdx.y;
     if (i0 >= L.nx || j >= L.ny) return;
@@ -274,9 +276,8 @@ static cudaError_t adj_step(const SweepArgs& a, const void* lam_in, void* lam_ou
     dim3 grid((unsigned)((L.nx + 32 * V - 1) / (32 * V)), (unsigned)((L.ny + BY - 1) / BY), 1);
     const int zchunk = adj_chunk((long long)grid.x * grid.y, L.nz);
     grid.z = (unsigned)((L.nz + zchunk - 1) / zchunk);
-    adjoint_vec_kernel<KIND, TF, TC, BY><<<grid, block, 0, s>>>(L, static_cast<const TF*>(lam_in),
-                                                                static_cast<TF*>(lam_out), C, zchunk);
-    return cudaGetLastError();
+    return launch_dependent(true, adjoint_vec_kernel<KIND, TF, TC, BY>, grid, block, 0, s, L, static_cast<const TF*>(lam_in),
+                            static_cast<TF*>(lam_out), C, zchunk);
 }
 
 cudaError_t adjoint_step(const SweepArgs& a, const void* lam_in, void* lam_out, cudaStream_t s) {

@@ -13,6 +13,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "pdl.cuh"
 #include "sweep_column.cuh"
 
 namespace stg {
@@ -35,6 +36,7 @@ __global__ void __launch_bounds__(32 * BY, (PlainCfg<KIND, TF, TC>::MINB))
 plain_sweep_kernel(Layout L, const TF* __restrict__ src, TF* __restrict__ dst, CoefPtrs<TC> C,
                    TF c0, TF c1, int zchunk) {
     constexpr int V = 16 / sizeof(TF);
+    dependent_begin();
     const int i0 = (blockIdx.x * 32 + threadIdx.x) * V;
     const int j = blockIdx.y * BY + threadIdx.y;
     if (i0 >= L.nx || j >= L.ny) return;
@@ -52,6 +54,7 @@ __global__ void __launch_bounds__(32 * BY) plain_async_kernel(Layout L, const TF
     constexpr int V = 16 / sizeof(TF);
     using Col = ColumnAsync<KIND, TF, TC, true, D>;
     extern __shared__ __align__(16) unsigned char plain_smem[];
+    dependent_begin();
     const int i0 = (blockIdx.x * 32 + threadIdx.x) * V;
     const int j = blockIdx.y * BY + threadIdx.y;
     if (i0 >= L.nx || j >= L.ny) return;
@@ -86,12 +89,15 @@ static int plain_slots(KernelT kernel, int threads, size_t smem = 0) {
 }
 
 // z chunks per column: minimise (waves of CTAs) x (planes per chunk + ring warm-up),
-// with chunks of at least 16 planes.
+// with chunks of at least 16 planes, or of any size while those would not fill the GPU once: a thread
+// walks its planes one memory latency after another (7-point constant FP64 64^3: 20.7 us a step in
+// chunks of 16 planes, 7.4 in chunks of one).
 static int plain_chunks(long long xy, int nz, int R, int slots) {
     if (slots <= 0) slots = 8 * 152;
     int best = 1;
     long long best_cost = -1;
-    const int maxchunks = (nz + 15) / 16 > 0 ? (nz + 15) / 16 : 1;
+    int maxchunks = (nz + 15) / 16 > 0 ? (nz + 15) / 16 : 1;
+    if (xy * maxchunks < slots) maxchunks = (int)(nz < slots / xy + 1 ? nz : slots / xy + 1);
     for (int n = 1; n <= maxchunks; ++n) {
         const int zc = (nz + n - 1) / n;
         const int nn = (nz + zc - 1) / zc;
@@ -124,20 +130,24 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
         const size_t smem = (size_t)D * 32 * BY * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R,
-                                         plain_slots<KIND, TF, TC>(kernel, 32 * BY, smem));
+        const int slots = plain_slots<KIND, TF, TC>(kernel, 32 * BY, smem);
+        const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots);
         const int zchunk = (L.nz + nchunks - 1) / nchunks;
-        kernel<<<dim3(gx, gy, (unsigned)nchunks), block, smem, s>>>(L, static_cast<const TF*>(src), static_cast<TF*>(dst),
-                                                                     C, (TF)a.c0, (TF)a.c1, zchunk);
-        return cudaGetLastError();
+        return launch_dependent(true, kernel, dim3(gx, gy, (unsigned)nchunks), block, smem, s, L,
+                                static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk);
     }
     auto kernel = plain_sweep_kernel<KIND, TF, TC, BY, PF>;
-    const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, plain_slots<KIND, TF, TC>(kernel, 32 * BY));
+    const int slots = plain_slots<KIND, TF, TC>(kernel, 32 * BY);
+    const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots);
     const int zchunk = (L.nz + nchunks - 1) / nchunks;
     dim3 grid(gx, gy, (unsigned)nchunks);
-    kernel<<<grid, block, 0, s>>>(L, static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1,
-                                  zchunk);
-    return cudaGetLastError();
+    // Set up beside the step before it (pdl.cuh), 64^3, us per step: 7-point constant FP64 20.7 -> 7.4, FP32
+    // 9.5 -> 2.8 (thinner chunks included), at 256^3 33.0 -> 31.0. Not FP64 sweeps of several waves: they
+    // are bound by the FP64 units, which the uneven second wave then loads unevenly (1 % slower at
+    // 203 x 250 x 141).
+    const bool early = sizeof(TF) == 4 || (long long)gx * gy * nchunks <= slots;
+    return launch_dependent(early, kernel, grid, block, 0, s, L, static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0,
+                            (TF)a.c1, zchunk);
 }
 
 cudaError_t plain_step(const SweepArgs& a, const void* src, void* dst, cudaStream_t s) {
