@@ -3,11 +3,11 @@
 // writes u_{t+1} once, so it moves 2*s_f + n_c*s_c bytes per LUP at best.
 //
 // Thread mapping: a warp covers 32 vectors of V = 16/sizeof(field) consecutive
-// x values (128-bit accesses); a CTA stacks BY warps along y; each thread walks
-// a chunk of z planes (sweep_column.cuh: register ring of the column's planes,
-// neighbours through L1/L2, coefficients with evict-first loads). The number
-// of z chunks is chosen from the kernel's occupancy so that the CTAs fill
-// whole waves of the GPU.
+// x values (128-bit accesses; FP64: fewer where a row is cut evenly, see launch_plain);
+// a CTA stacks BY rows along y; each thread walks a chunk of z planes
+// (sweep_column.cuh: register ring of the column's planes, neighbours through L1/L2,
+// coefficients with evict-first loads). The number of z chunks is chosen from the
+// kernel's occupancy so that the CTAs fill whole waves of the GPU.
 #include <stdint.h>
 
 #include <mutex>
@@ -22,9 +22,14 @@ namespace stg {
 // allocation must allow (MINB), chosen by measurement on GB300. The constant-coefficient
 // sweep has a single HBM stream per thread and wants loads in flight; the variable ones
 // issue n_c + 1 streaming loads per plane already and are limited by the registers their
-// coefficient vectors take (the 25-point BF16 / FP64 sweeps double their speed at 2 CTAs).
+// coefficient vectors take (the 25-point BF16 / FP64 sweeps double their speed at 2 CTAs). The
+// constant FP64 sweep is bound by the FP64 pipe and forms 3 of its 7 operations on the integer pipes
+// (upd7c_soft): 512^3 79.6 -> 120 GLUP/s, 64^3 36 -> 52, 203 x 250 x 141 49 -> 88 (cut evenly, see
+// launch_plain). GLUP/s at 512^3 by operations moved: the product 97, and one pair sum 102, two 120, three 97
+// (more integer work than the pipe saved); registers: 4 CTAs 120, 3 118, 2 110, 5 (spills) 119.
 template <int KIND, typename TF, typename TC> struct PlainCfg { static constexpr int PF = 1, MINB = 1; };
 template <typename TF> struct PlainCfg<K7C, TF, TF> { static constexpr int PF = 3, MINB = 5; };
+template <> struct PlainCfg<K7C, double, double> { static constexpr int PF = 1, MINB = 4; };
 template <> struct PlainCfg<K7V, float, float> { static constexpr int PF = 0, MINB = 3; };
 template <> struct PlainCfg<K7V, double, double> { static constexpr int PF = 0, MINB = 3; };
 template <> struct PlainCfg<K25V, float, float> { static constexpr int PF = 0, MINB = 1; };
@@ -34,16 +39,17 @@ template <> struct PlainCfg<K25V, double, double> { static constexpr int PF = 1,
 template <int KIND, typename TF, typename TC, int BY, int PF>
 __global__ void __launch_bounds__(32 * BY, (PlainCfg<KIND, TF, TC>::MINB))
 plain_sweep_kernel(Layout L, const TF* __restrict__ src, TF* __restrict__ dst, CoefPtrs<TC> C,
-                   TF c0, TF c1, int zchunk) {
+                   TF c0, TF c1, int zchunk, int width) {
     constexpr int V = 16 / sizeof(TF);
     dependent_begin();
-    const int i0 = (blockIdx.x * 32 + threadIdx.x) * V;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    if (i0 >= L.nx || j >= L.ny) return;
+    const int ty = (int)threadIdx.x / width;
+    const int i0 = (blockIdx.x * width + (threadIdx.x - ty * width)) * V;
+    const int j = blockIdx.y * BY + ty;
+    if (i0 >= L.nx || j >= L.ny || ty >= BY) return;
     const int k0 = blockIdx.z * zchunk;
     const int k1 = min(L.nz, k0 + zchunk);
     if (k0 >= k1) return;
-    sweep_column<KIND, TF, TC, PF, true>(L, src, dst, C, c0, c1, i0, j, k0, k1);
+    sweep_column<KIND, TF, TC, PF, true, false, KIND == K7C && sizeof(TF) == 8>(L, src, dst, C, c0, c1, i0, j, k0, k1);
 }
 
 // The plain sweep with every load of a plane copied D planes ahead into per-thread shared-memory
@@ -75,17 +81,18 @@ __global__ void __launch_bounds__(32 * BY) plain_async_kernel(Layout L, const TF
 template <int KIND, typename TF, typename TC, typename KernelT>
 static int plain_slots(KernelT kernel, int threads, size_t smem = 0) {
     static std::mutex mu;
-    static int cached[64] = {0};
+    static int cached[64][33] = {};  // by device and warps
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     std::lock_guard<std::mutex> lock(mu);
-    if (cached[dev] == 0) {
+    int& c = cached[dev][threads / 32];
+    if (c == 0) {
         int sms = 0, per = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess) return 0;
-        cached[dev] = sms * (per > 0 ? per : 1);
+        c = sms * (per > 0 ? per : 1);
     }
-    return cached[dev];
+    return c;
 }
 
 // z chunks per column: minimise (waves of CTAs) x (planes per chunk + ring warm-up),
@@ -137,7 +144,13 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
                                 static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk);
     }
     auto kernel = plain_sweep_kernel<KIND, TF, TC, BY, PF>;
-    const int slots = plain_slots<KIND, TF, TC>(kernel, 32 * BY);
+    // Vectors of a row per CTA. FP64 (bound by its pipe, which idle lanes hold as well): the row is cut
+    // evenly and the CTA's rows follow one another in its warps, GLUP/s at 203 x 250 x 141: 7-point
+    // constant 46 -> 52, 7-point variable 59 -> 63, 25-point (130 x 200 x 162) 14.6 -> 19.0. FP32 (bound
+    // by HBM): a row per warp; 25-point 303 x 150 x 141 92.0 GLUP/s, cut evenly 90.8.
+    const int width = sizeof(TF) == 8 ? (L.nx + (int)gx * V - 1) / ((int)gx * V) : 32;
+    const int threads = (width * BY + 31) / 32 * 32;
+    const int slots = plain_slots<KIND, TF, TC>(kernel, threads);
     const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots);
     const int zchunk = (L.nz + nchunks - 1) / nchunks;
     dim3 grid(gx, gy, (unsigned)nchunks);
@@ -146,8 +159,8 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
     // are bound by the FP64 units, which the uneven second wave then loads unevenly (1 % slower at
     // 203 x 250 x 141).
     const bool early = sizeof(TF) == 4 || (long long)gx * gy * nchunks <= slots;
-    return launch_dependent(early, kernel, grid, block, 0, s, L, static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0,
-                            (TF)a.c1, zchunk);
+    return launch_dependent(early, kernel, grid, dim3((unsigned)threads), 0, s, L, static_cast<const TF*>(src),
+                            static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk, width);
 }
 
 cudaError_t plain_step(const SweepArgs& a, const void* src, void* dst, cudaStream_t s) {

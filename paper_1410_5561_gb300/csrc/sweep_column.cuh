@@ -18,6 +18,7 @@
 // it only after acquiring their completion flags.
 #pragma once
 #include "internal.h"
+#include "soft64.cuh"
 
 namespace stg {
 
@@ -107,6 +108,42 @@ template <> struct CoefLds<__nv_bfloat16, 4> {
     }
 };
 
+// Listing 1 for V points in FP64, the operations of upd7c in their order, with the product and the y
+// and z pair sums formed on the integer pipes: 4 of 7 operations are left to the FP64 pipe. Where the
+// integer forms do not take one of the points (those past the row's end, from `left` on, do not
+// count), all V are formed by the FP64 pipe, so a field with many zeros costs what it did without.
+template <int V>
+__device__ __forceinline__ void upd7c_soft(double c0, double c1, const double* v, const double* xp, const double* xm,
+                                           const double* yp, const double* ym, const double* zp, const double* zm,
+                                           int left, double* out) {
+    using A = Ar<double>;
+    const SoftFactor f0(c0);
+    double r[V], sy[V], sz[V];
+    uint32_t bad = 0;
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+        uint32_t b = 0;
+        r[e] = soft_mul(f0, v[e], b);
+        sy[e] = soft_add(yp[e], ym[e], b);
+        sz[e] = soft_add(zp[e], zm[e], b);
+        if (e < left) bad |= b;
+    }
+    if (bad) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            r[e] = A::mul(c0, v[e]);
+            sy[e] = A::add(yp[e], ym[e]);
+            sz[e] = A::add(zp[e], zm[e]);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+        r[e] = A::fma(c1, A::add(xp[e], xm[e]), r[e]);
+        r[e] = A::fma(c1, sy[e], r[e]);
+        out[e] = A::fma(c1, sz[e], r[e]);
+    }
+}
+
 // The column walk as a resumable state: begin() loads the planes below the first
 // plane, plane() updates the next plane (planes in increasing order, starting at
 // begin's k0; no plane at or beyond k1 is loaded). Loads reach R + PF planes above
@@ -117,7 +154,7 @@ template <> struct CoefLds<__nv_bfloat16, 4> {
 // ring position 0 and array 0; cstep: bytes between consecutive (position, array) slots), so
 // the copies in flight hold shared memory instead of registers. Each thread reads only the
 // slots it filled, after its own cp.async.wait_group: no CTA barrier is needed.
-template <int KIND, typename TF, typename TC, int PF, bool COEF_STREAM, bool COHERENT, int CP = 0>
+template <int KIND, typename TF, typename TC, int PF, bool COEF_STREAM, bool COHERENT, int CP = 0, bool SOFT = false>
 struct Column {
     static constexpr int R = KindTraits<KIND>::R;
     static constexpr int NC = KindTraits<KIND>::NC;
@@ -205,8 +242,11 @@ struct Column {
         }
 
         Vec<TF, V> out;
+        if constexpr (SOFT)
+            upd7c_soft<V>(c0, c1, ring[R].v, xl + J * V + 1, xl + J * V - 1, yp[0].v, ym[0].v, ring[R + 1].v, ring[R - 1].v,
+                          L.nx - i0, out.v);
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
+        for (int e = 0; e < V && !SOFT; ++e) {
             const int xc = J * V + e;
             if constexpr (KIND == K7C) {
                 out.v[e] = upd7c<TF>(c0, c1, ring[R].v[e], xl[xc + 1], xl[xc - 1], yp[0].v[e],
@@ -392,10 +432,10 @@ struct ColumnAsync {
     }
 };
 
-template <int KIND, typename TF, typename TC, int PF, bool COEF_STREAM, bool COHERENT = false>
+template <int KIND, typename TF, typename TC, int PF, bool COEF_STREAM, bool COHERENT = false, bool SOFT = false>
 __device__ __forceinline__ void sweep_column(const Layout& L, const TF* __restrict__ src, TF* __restrict__ dst,
                                              const CoefPtrs<TC>& C, TF c0, TF c1, int i0, int j, int k0, int k1) {
-    Column<KIND, TF, TC, PF, COEF_STREAM, COHERENT> col;
+    Column<KIND, TF, TC, PF, COEF_STREAM, COHERENT, 0, SOFT> col;
     col.begin(L, src, i0, j, k0, k1);
     for (int k = k0; k < k1; ++k) col.plane(L, src, dst, C, c0, c1, i0, k);
 }

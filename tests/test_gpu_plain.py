@@ -132,3 +132,33 @@ def test_prefetched_plain_sweep_is_bitwise_equal(kind, shape, fdt, cdt, T):
     b.set_tuning("plain", Tuning(0, 2, 0, 0))
     b.run(T)
     assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 9, 5), (63, 8, 4), (64, 7, 3), (66, 17, 9), (203, 12, 20)])
+@pytest.mark.parametrize("c0", [0.4, -3.0, 0.0, 5e-324, 1e300])
+def test_fp64_constant_sweep_takes_every_value(shape, c0):
+    """The FP64 constant sweep forms some operations on the integer pipes: its bits are those of the same
+    operations, each rounded to nearest (the x, y and z pair sums, a product, three fused sums), for
+    fields with zeros of both signs, subnormals, cancelling neighbours, infinities and NaN."""
+    import torch
+    from paper_1410_5561_gb300.stencil import Stencil, Tuning
+    nx, ny, nz = shape
+    g = torch.Generator().manual_seed(nx + 7 * ny)
+    u = torch.rand((nz, ny, nx), generator=g, dtype=torch.float64) * 2 - 1
+    pick = torch.randint(0, 40, (nz, ny, nx), generator=g)
+    for i, v in enumerate([0.0, -0.0, 5e-324, -2.0 ** -1023, 2.0 ** -970, 2.0 ** 1023, -1.5 * 2.0 ** 1023, 1.0, -1.0,
+                           float("inf"), float("nan")]):
+        u[pick == i] = v
+    for T in (1, 2):
+        out = []
+        for scheme, tn in (("plain", None), ("wavefront", Tuning(8, 4, 4, 0))):
+            s = Stencil("7pt_const", nx, ny, nz, dtype=torch.float64)
+            s.set_coeffs(scalars=(c0, 0.1))
+            s.set_tuning(scheme, tn)
+            s.set_field(u.cuda(), halo=0.0)
+            s.run(T)
+            out.append(s.get_field())
+        a, b = out
+        assert torch.equal(torch.isnan(a), torch.isnan(b))
+        ok = ~torch.isnan(a)
+        assert torch.equal(a[ok].view(torch.int64), b[ok].view(torch.int64))
