@@ -52,13 +52,14 @@ struct AdjSteps {
 };
 
 // FP32 -> FP64 without the FP64 pipe, which also does the hardware conversion and already bounds
-// this kernel: N values at once, by integer operations where all of them are normal numbers or zeros (the
+// this kernel: N values at once, by integer operations where all of them are normal numbers or, with ZEROS, zeros (the
 // magnitude times 2^29 as a 64-bit integer is the FP64 significand and exponent field, short of
 // the difference of the two exponent biases), else by the hardware conversion. Exact either way. Zeros
 // are every cell next to the halo and every lane past a ragged row's end: left to the hardware they
 // took whole warps there (training step, 25-point BF16 203 x 250 x 141 T = 12: 7.1 -> 5.8 ms, 7-point FP32
-// 250 x 220 x 180 T = 20: 8.8 -> 7.2 ms).
-template <int N>
+// 250 x 220 x 180 T = 20: 8.8 -> 7.2 ms). Not for the 25-point stencil on rows of whole vectors: its weights
+// are pair sums, none of them zero for a halo alone, and the two operations more per value cost 1 %.
+template <int N, bool ZEROS>
 struct Widen {
     double d[N];
     __device__ __forceinline__ explicit Widen(const float* x) {
@@ -66,14 +67,14 @@ struct Widen {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             a[i] = __float_as_uint(x[i]) & 0x7fffffffu;
-            lo = min(lo, a[i] - 1u);  // zeros become the largest value
+            lo = min(lo, ZEROS ? a[i] - 1u : a[i]);  // (zeros become the largest value)
             hi = max(hi, a[i]);
         }
-        if (lo >= 0x007fffffu && hi < 0x7f800000u) {
+        if (lo >= (ZEROS ? 0x007fffffu : 0x00800000u) && hi < 0x7f800000u) {
 #pragma unroll
             for (int i = 0; i < N; ++i) {
                 const unsigned long long w = (unsigned long long)a[i] * (1u << 29) + (896ull << 52);
-                const unsigned h = a[i] != 0u ? (unsigned)(w >> 32) : 0u;  // (the low half of a zero is zero)
+                const unsigned h = !ZEROS || a[i] != 0u ? (unsigned)(w >> 32) : 0u;  // (the low half of a zero is zero)
                 d[i] = __hiloint2double((int)(h | (__float_as_uint(x[i]) & 0x80000000u)), (int)(unsigned)w);
             }
         } else {
@@ -91,7 +92,7 @@ struct Widen {
 // arrays, 256^3, 40 steps). With hardware conversions of the weights on the same pipe it took
 // 34.0 ms, with Widen 19.4, at three CTAs per SM (168 registers, 24 bytes spilled) 17.6; vectors of
 // two points (more warps, but twice the loads) 29.6.
-template <int KIND, typename TF, int V, int NT>
+template <int KIND, typename TF, int V, int NT, bool ZEROS>
 __global__ void __launch_bounds__(NT, 3) adjoint_grad_kernel(Layout L, AdjSteps<TF> S, int nsteps, AdjGrad G, int zchunk) {
     constexpr int R = KindTraits<KIND>::R;
     constexpr int NC = KindTraits<KIND>::NC;
@@ -137,12 +138,12 @@ __global__ void __launch_bounds__(NT, 3) adjoint_grad_kernel(Layout L, AdjSteps<
 #pragma unroll
                 for (int e = 0; e < V; ++e) ux[(q + J) * V + e] = wu.v[e];
             }
-            const Widen<V> lam(lv.v);
+            const Widen<V, ZEROS> lam(lv.v);
             // weight of array m: 7-point C0 u(p), C(2a+1) u(p + e_a), C(2a+2) u(p - e_a);
             // 25-point C00 u(p), C(3(d-1)+a+1) (u(p + d e_a) + u(p - d e_a)), the pair sum
             // in the field precision as the forward step forms it
             {
-                const Widen<V> w(ux + J * V);
+                const Widen<V, ZEROS> w(ux + J * V);
 #pragma unroll
                 for (int e = 0; e < V; ++e) gv[0][e] = __fma_rn(lam.d[e], w.d[e], gv[0][e]);
             }
@@ -170,7 +171,7 @@ __global__ void __launch_bounds__(NT, 3) adjoint_grad_kernel(Layout L, AdjSteps<
                 }
                 if constexpr (KIND == K7V) {
                     // C(2a+1) weighs u(p + e_a), C(2a+2) weighs u(p - e_a)
-                    const Widen<3 * V> wp(&up[0][0]), wm(&um[0][0]);
+                    const Widen<3 * V, ZEROS> wp(&up[0][0]), wm(&um[0][0]);
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(NT, 3) adjoint_grad_kernel(Layout L, AdjSteps<
                     for (int a = 0; a < 3; ++a)
 #pragma unroll
                         for (int e = 0; e < V; ++e) up[a][e] = A::add(up[a][e], um[a][e]);
-                    const Widen<3 * V> w(&up[0][0]);
+                    const Widen<3 * V, ZEROS> w(&up[0][0]);
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
                         const int m = 3 * (d - 1) + a + 1;
@@ -235,7 +236,8 @@ static cudaError_t adj_grads(const Layout& L, const void* const* lam, const void
             S.lam[g] = static_cast<const TF*>(lam[g0 + g]);
             S.u[g] = static_cast<const TF*>(u[g0 + g]);
         }
-        adjoint_grad_kernel<KIND, TF, V, NT><<<grid, NT, 0, s>>>(L, S, ng, G, zchunk);
+        if (KIND == K25V && L.nx % V == 0) adjoint_grad_kernel<KIND, TF, V, NT, KIND != K25V><<<grid, NT, 0, s>>>(L, S, ng, G, zchunk);
+        else adjoint_grad_kernel<KIND, TF, V, NT, true><<<grid, NT, 0, s>>>(L, S, ng, G, zchunk);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
