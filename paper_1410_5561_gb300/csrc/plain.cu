@@ -56,19 +56,19 @@ plain_sweep_kernel(Layout L, const TF* __restrict__ src, TF* __restrict__ dst, C
 // slots (ColumnAsync): the copies in flight hold shared memory, not registers.
 template <int KIND, typename TF, typename TC, int BY, int D>
 __global__ void __launch_bounds__(32 * BY) plain_async_kernel(Layout L, const TF* __restrict__ src, TF* __restrict__ dst,
-                                                              CoefPtrs<TC> C, TF c0, TF c1, int zchunk) {
+                                                              CoefPtrs<TC> C, TF c0, TF c1, int zchunk, int width) {
     constexpr int V = 16 / sizeof(TF);
     using Col = ColumnAsync<KIND, TF, TC, true, D>;
     extern __shared__ __align__(16) unsigned char plain_smem[];
     dependent_begin();
-    const int i0 = (blockIdx.x * 32 + threadIdx.x) * V;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    if (i0 >= L.nx || j >= L.ny) return;
+    const int ty = (int)threadIdx.x / width;
+    const int i0 = (blockIdx.x * width + (threadIdx.x - ty * width)) * V;
+    const int j = blockIdx.y * BY + ty;
+    if (i0 >= L.nx || j >= L.ny || ty >= BY) return;
     const int k0 = blockIdx.z * zchunk;
     const int k1 = min(L.nz, k0 + zchunk);
     if (k0 >= k1) return;
-    constexpr int NT = 32 * BY;
-    const int tid = (int)(threadIdx.y * 32 + threadIdx.x);
+    const int NT = (int)blockDim.x, tid = (int)threadIdx.x;
     const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(plain_smem);
     Col col;
     col.begin(L, src, C, i0, j, k0, k1, s0 + (uint32_t)(tid * 16), (uint32_t)(NT * 16),
@@ -98,13 +98,15 @@ static int plain_slots(KernelT kernel, int threads, size_t smem = 0) {
 // z chunks per column: minimise (waves of CTAs) x (planes per chunk + ring warm-up),
 // with chunks of at least 16 planes, or of any size while those would not fill the GPU once: a thread
 // walks its planes one memory latency after another (7-point constant FP64 64^3: 20.7 us a step in
-// chunks of 16 planes, 7.4 in chunks of one).
-static int plain_chunks(long long xy, int nz, int R, int slots) {
+// chunks of 16 planes, 7.4 in chunks of one). thin: the CTAs up to which chunks get thinner (0: slots; more
+// CTAs than that fit where they are narrower, but thinner chunks then only repeat more first planes).
+static int plain_chunks(long long xy, int nz, int R, int slots, int thin = 0) {
     if (slots <= 0) slots = 8 * 152;
+    if (thin <= 0) thin = slots;
     int best = 1;
     long long best_cost = -1;
     int maxchunks = (nz + 15) / 16 > 0 ? (nz + 15) / 16 : 1;
-    if (xy * maxchunks < slots) maxchunks = (int)(nz < slots / xy + 1 ? nz : slots / xy + 1);
+    if (xy * maxchunks < thin) maxchunks = (int)(nz < thin / xy + 1 ? nz : thin / xy + 1);
     for (int n = 1; n <= maxchunks; ++n) {
         const int zc = (nz + n - 1) / n;
         const int nn = (nz + zc - 1) / zc;
@@ -127,21 +129,27 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
     if (L.nx == 0 || L.ny == 0 || L.nz == 0) return cudaSuccess;
     CoefPtrs<TC> C{};
     for (int m = 0; m < KindTraits<KIND>::NC; ++m) C.c[m] = static_cast<const TC*>(a.coef[m]);
-    dim3 block(32, BY);
     unsigned gx = (unsigned)((L.nx + 32 * V - 1) / (32 * V));
     unsigned gy = (unsigned)((L.ny + BY - 1) / BY);
     if (a.plain_prefetch == 2) {
         constexpr int D = 2;
         using Col = ColumnAsync<KIND, TF, TC, true, D>;
         auto kernel = plain_async_kernel<KIND, TF, TC, BY, D>;
-        const size_t smem = (size_t)D * 32 * BY * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // Rows of more than one CTA are cut evenly, so that no CTA has its slots for a few lanes: 25-point BF16,
+        // GLUP/s, 203 x 250 x 141 116 -> 120, 130 x 200 x 90 87 -> 101, 140 x 64 x 300 89 -> 106. Not rows of one CTA,
+        // where a narrower one only has fewer warps: 64^3 56 -> 39-45, 33 x 500 x 100 47 -> 44.
+        const int width = gx > 1 ? (L.nx + (int)gx * V - 1) / ((int)gx * V) : 32;
+        const int threads = (width * BY + 31) / 32 * 32;
+        const size_t smem = (size_t)D * threads * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
+        constexpr int FULL = D * 32 * BY * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FULL);
         if (e != cudaSuccess) return e;
-        const int slots = plain_slots<KIND, TF, TC>(kernel, 32 * BY, smem);
-        const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots);
+        const int slots = plain_slots<KIND, TF, TC>(kernel, threads, smem);
+        const int thin = plain_slots<KIND, TF, TC>(kernel, 32 * BY, FULL);
+        const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots, thin);
         const int zchunk = (L.nz + nchunks - 1) / nchunks;
-        return launch_dependent(true, kernel, dim3(gx, gy, (unsigned)nchunks), block, smem, s, L,
-                                static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk);
+        return launch_dependent(true, kernel, dim3(gx, gy, (unsigned)nchunks), dim3((unsigned)threads), smem, s, L,
+                                static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk, width);
     }
     auto kernel = plain_sweep_kernel<KIND, TF, TC, BY, PF>;
     // Vectors of a row per CTA. FP64 (bound by its pipe, which idle lanes hold as well): the row is cut
