@@ -65,6 +65,8 @@ struct TileMeta {
     int vlo[MAXLV];                    // first computed ring vector
     int xlo[MAXLV], xhi[MAXLV];        // computed x range (interior coordinates)
     int ldlo[MAXLV], ldhi[MAXLV];      // ring vectors loaded for this level's input
+    // Rows of tasks and items are relative to row b D + R t0, the first one that the diamond could
+    // own at its first level: they then fit 16 bits for any grid (absolute rows do not beyond 32767).
     short tl[MAXTASK], ty[MAXTASK];    // load / fill tasks for interior planes
     unsigned char tfill[MAXTASK];
     int tpre[MAXTASK + 1];             // vectors of tasks [0, i): a task moves one ring row
@@ -319,6 +321,7 @@ __device__ __forceinline__ void run_tile(const GridArgs<TF, TC>& P, const int k,
         M.Lt = Lt;
         M.t0 = tlo;
         int off = 0, ntask = 0, nitem = 0;
+        const int yb = b * D + R * tlo;
         for (int l = 0; l < Lt; ++l) {
             int lo, hi;
             level_rows(D, R, Ny, a, b, tlo + l, lo, hi);
@@ -359,7 +362,7 @@ __device__ __forceinline__ void run_tile(const GridArgs<TF, TC>& P, const int k,
                     const bool computed = !halo_row && y >= blo && y < bhi;
                     if (computed || ntask >= MAXTASK) continue;
                     M.tl[ntask] = (short)l;
-                    M.ty[ntask] = (short)y;
+                    M.ty[ntask] = (short)(y - yb);
                     M.tfill[ntask] = halo_row ? 1 : 0;
                     ++ntask;
                 }
@@ -367,7 +370,7 @@ __device__ __forceinline__ void run_tile(const GridArgs<TF, TC>& P, const int k,
                 for (int y = lo; y < hi; y += RB)
                     for (int c = 0; c < nch && nitem < MAXITEM; ++c) {
                         M.il[nitem] = (short)l;
-                        M.iy[nitem] = (short)y;
+                        M.iy[nitem] = (short)(y - yb);
                         M.ich[nitem] = (unsigned char)c;
                         M.inr[nitem] = (unsigned char)(hi - y < RB ? hi - y : RB);
                         ++nitem;
@@ -395,6 +398,7 @@ __device__ __forceinline__ void run_tile(const GridArgs<TF, TC>& P, const int k,
     __syncthreads();
     const int Lt = M.Lt;
     if (Lt == 0) return;
+    const int yb = b * D + R * M.t0;
     const TF hv = P.halo;
     uint32_t tok = 0;  // barrier token of the fast path's shared-memory loads
     if constexpr (PERSIST) {
@@ -421,7 +425,7 @@ __device__ __forceinline__ void run_tile(const GridArgs<TF, TC>& P, const int k,
         const int id = warp + kk * NW;
         I.valid = id < M.nitem;
         if (!I.valid) continue;
-        const int l = M.il[id], y0 = M.iy[id];
+        const int l = M.il[id], y0 = yb + M.iy[id];
         I.nr = M.inr[id];
         const int nlo = M.nlo[l];
         I.PS = (M.nhi[l] - nlo) * Xs;
@@ -500,7 +504,7 @@ __device__ __forceinline__ void run_tile(const GridArgs<TF, TC>& P, const int k,
             pa_sl[j] = 0;
             if (!pa_ok[j]) continue;
             while (M.tpre[ti + 1] <= q) ++ti;
-            const int l = M.tl[ti], y = M.ty[ti];
+            const int l = M.tl[ti], y = yb + M.ty[ti];
             const int nlo = M.nlo[l];
             const int c = M.ldlo[l] + (q - M.tpre[ti]);
             pa_psb[j] = (uint32_t)((M.nhi[l] - nlo) * Xs * (int)sizeof(TF));
@@ -582,7 +586,7 @@ __device__ __forceinline__ void run_tile(const GridArgs<TF, TC>& P, const int k,
         }
         for (int q = tid + KT * NT, ti = 0; q < npair; q += NT) {
             while (M.tpre[ti + 1] <= q) ++ti;
-            const int l = M.tl[ti], y = M.ty[ti];
+            const int l = M.tl[ti], y = yb + M.ty[ti];
             const int nlo = M.nlo[l];
             const int c = M.ldlo[l] + (q - M.tpre[ti]);
             const int PS = (M.nhi[l] - nlo) * Xs;

@@ -270,3 +270,14 @@ def test_model_guided_tuner_times_three_and_keeps_the_best():
     torch.cuda.synchronize()
     mine = tuner._time_run(s, T, 3)
     assert mine <= 1.10 * best_full, (tn, mine, full, best_full)
+
+
+@pytest.mark.parametrize("kind,fdt,tn,T", [
+    ("7pt_const", "f32", Tuning(8, 2, 16, 4), 9),
+    ("7pt_var", "f32", Tuning(4, 1, 8, 4), 6),
+    ("25pt_var", "f64", Tuning(8, 1, 8, 4), 3),
+])
+def test_blocked_rows_beyond_16_bits(kind, fdt, tn, T):
+    """A grid of more than 32767 rows: the tile's table of rows holds them all."""
+    p = Problem(kind, 3, 33500, 4, fdt=fdt, seed=21, halo=0.5)
+    assert np.array_equal(_run(p, T, "plain"), _run(p, T, "blocked", tn))
