@@ -34,12 +34,11 @@
 // 7-point variable 384^3: FP32 200 -> 425 (HBM at 5.2 TB/s, 13 bytes per update), BF16 253 -> 484
 // (issue and latency of the widening).
 #pragma once
-#include <limits.h>
-
 #include <type_traits>
 
 #include "internal.h"
 #include "overlap.h"
+#include "overlap_rings.h"
 #include "tma.cuh"
 
 namespace stg {
@@ -142,11 +141,6 @@ struct OvCfg {
     static_assert(PLANEB % 128 == 0 && PUB0 % 16 == 0, "box destinations stay 128-byte aligned");
 };
 
-// The copy rings' positions, carried from one tile to the next in shared memory: slot and phase of
-// the next plane.
-struct OvRings {
-    int fs, cs, fp, cp;
-};
 // A value that is the same in every lane, told to the compiler (it then lives in uniform registers:
 // 1892 against 1740 GLUP/s at 1024^3 for the warp index alone).
 __device__ __forceinline__ int ov_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
@@ -195,13 +189,17 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
                             z + 1, cbar + 8 * slot);
         }
     };
-    const OvRings r0{ov_uniform(ring->fs), ov_uniform(ring->cs), ov_uniform(ring->fp), ov_uniform(ring->cp)};
-    if (threadIdx.x == 0) {
+    const OvRings r0{ov_uniform(ring->fs), ov_uniform(ring->cs), ov_uniform(ring->fp), ov_uniform(ring->cp),
+                     ov_uniform(ring->lost)};
+    // iteration in which a copy did not arrive in time (the results are invalid): no more copies
+    // are issued and no more waits made, in this tile and in the CTA's later ones (overlap_rings.h)
+    int lost = ov_lost_before(r0, s_begin);
+    if (threadIdx.x == 0 && lost == OV_NOT_LOST) {
         for (int p = 0; p < PD; ++p)
-            if (s_begin + p < zl) copy(s_begin + p, (r0.fs + p) % S::RING);
+            if (s_begin + p < zl) copy(s_begin + p, ov_slot(r0.fs, p, S::RING));
         if constexpr (NC > 0)
             for (int p = 0; p < CR - 1; ++p)
-                if (cb + p < ce) ccopy(cb + p, (r0.cs + p) % CR);
+                if (cb + p < ce) ccopy(cb + p, ov_slot(r0.cs, p, CR));
     }
     const uint32_t own = s0 + (uint32_t)((w * RB + 1) * S::ROWB + lane * 16);
     const uint32_t cown = s0 + (uint32_t)(S::COEF0 + w * RB * S::CROWB + (S::CX0 + lane * 4) * (int)sizeof(TC));
@@ -247,11 +245,8 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
     // coefficient slot of plane s - 1 (level 0's) and its phase, from plane cb on
     int cl = r0.cs;
     uint32_t cph = (uint32_t)r0.cp;
-    // iteration in which a copy did not arrive in time (the results are invalid): no more copies
-    // are issued and no more waits made
-    int lost = INT_MAX;
     auto arrived = [&](uint32_t b, uint32_t phase, int s) {
-        if (!mbar_test(b, phase) && lost == INT_MAX && !mbar_wait(b, phase, status)) lost = s;
+        if (!mbar_test(b, phase) && lost == OV_NOT_LOST && !mbar_wait(b, phase, status)) lost = s;
     };
 
     // STEADY: every plane of the iteration is a real plane and is stored. The other iterations
@@ -262,7 +257,7 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
         constexpr bool STEADY = decltype(steadyc)::value;
         constexpr int ZM = PH % 3, ZC = (PH + 1) % 3, ZP = (PH + 2) % 3;
         const bool cnow = NC > 0 && (STEADY || (s - 1 >= cb && s - 1 < ce));
-        if (threadIdx.x == 0 && lost == INT_MAX) {
+        if (threadIdx.x == 0 && lost == OV_NOT_LOST) {
             if (s + PD < zl) copy(s + PD, slf);
             if (NC > 0) {
                 // the slot of plane s - 2, read in the iteration before: plane s - 2 + CR (those up to
@@ -425,18 +420,19 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
     if (HL < H || mode == 2) walk(std::integral_constant<int, 2>{});
     else if (mode == 1) walk(std::integral_constant<int, 1>{});
     else walk(std::integral_constant<int, 0>{});
-    if (threadIdx.x == 0 && lost != INT_MAX) {
-        // the copies still in flight end before the CTA goes on (bounded): the last one of every slot
-        const int fl = min(zl, lost + PD + 1) - 1 - s_begin, cf = min(ce, max(cb + CR - 1, lost + CR - 1)) - 1 - cb;
-        for (int p = max(0, fl - S::RING + 1); p <= fl; ++p)
-            mbar_wait(bar + 8 * ((r0.fs + p) % S::RING), (uint32_t)(r0.fp ^ ((r0.fs + p) / S::RING & 1)), status);
-        for (int p = max(0, cf - CR + 1); NC > 0 && p <= cf; ++p)
-            mbar_wait(cbar + 8 * ((r0.cs + p) % CR), (uint32_t)(r0.cp ^ ((r0.cs + p) / CR & 1)), status);
-    }
     if (threadIdx.x == 0) {
+        int nf = zl - s_begin, nc = ce > cb ? ce - cb : 0;
+        if (lost != OV_NOT_LOST && !r0.lost) {
+            // the copies still in flight end before the CTA goes on (bounded): the last one of every slot
+            nf = ov_issued_fields(s_begin, zl, lost, PD);
+            nc = ov_issued_coefs(cb, ce, lost, CR);
+            for (int p = max(0, nf - S::RING); p < nf; ++p)
+                mbar_wait(bar + 8 * ov_slot(r0.fs, p, S::RING), (uint32_t)ov_phase(r0.fs, r0.fp, p, S::RING), status);
+            for (int p = max(0, nc - CR); NC > 0 && p < nc; ++p)
+                mbar_wait(cbar + 8 * ov_slot(r0.cs, p, CR), (uint32_t)ov_phase(r0.cs, r0.cp, p, CR), status);
+        }
         // read by every thread after the barrier that follows the tile
-        const int nf = r0.fs + zl - s_begin, nc = r0.cs + ce - cb;
-        *ring = OvRings{nf % S::RING, NC > 0 ? nc % CR : 0, r0.fp ^ (nf / S::RING & 1), NC > 0 ? r0.cp ^ (nc / CR & 1) : 0};
+        *ring = ov_rings_after(r0, nf, NC > 0 ? nc : 0, S::RING, CR, lost != OV_NOT_LOST);
     }
 }
 
@@ -484,7 +480,7 @@ __global__ void __launch_bounds__(NW * 32, 1) overlap_kernel(const __grid_consta
     if (threadIdx.x == 0) {
         for (int p = 0; p < S::RING + CR; ++p) mbar_init(s0 + S::BAR0 + 8 * p, 1);
         mbar_init_fence();
-        s_ring = OvRings{0, 0, 0, 0};
+        s_ring = OvRings{0, 0, 0, 0, 0};
     }
     const int tiles = G.ntx * G.nty * G.ntz, items = tiles * G.passes;
     int next = 0;  // thread 0: the item to do next
@@ -549,7 +545,7 @@ __global__ void __launch_bounds__(NW * 32, 1) overlap_batch_kernel(const OvBatch
     if (threadIdx.x == 0) {
         for (int p = 0; p < S::RING + CR; ++p) mbar_init(s0 + S::BAR0 + 8 * p, 1);
         mbar_init_fence();
-        s_ring = OvRings{0, 0, 0, 0};
+        s_ring = OvRings{0, 0, 0, 0, 0};
     }
     const OvCtl C{B.status, B.never, B.head, B.done, B.spin_limit, -1};
     int next = 0;  // thread 0: the item to do next
