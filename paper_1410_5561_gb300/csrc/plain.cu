@@ -10,9 +10,8 @@
 // kernel's occupancy so that the CTAs fill whole waves of the GPU.
 #include <stdint.h>
 
-#include <mutex>
-
 #include "internal.h"
+#include "occupancy.h"
 #include "pdl.cuh"
 #include "sweep_column.cuh"
 
@@ -76,25 +75,6 @@ __global__ void __launch_bounds__(32 * BY) plain_async_kernel(Layout L, const TF
     for (int k = k0; k < k1; ++k) col.plane(L, src, dst, C, c0, c1, i0, k);
 }
 
-// Resident CTAs per SM of one kernel instantiation times the SM count, per device
-// (one cache per instantiation: the template arguments name the kernel).
-template <int KIND, typename TF, typename TC, typename KernelT>
-static int plain_slots(KernelT kernel, int threads, size_t smem = 0) {
-    static std::mutex mu;
-    static int cached[64][33] = {};  // by device and warps
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    std::lock_guard<std::mutex> lock(mu);
-    int& c = cached[dev][threads / 32];
-    if (c == 0) {
-        int sms = 0, per = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess) return 0;
-        c = sms * (per > 0 ? per : 1);
-    }
-    return c;
-}
-
 // z chunks per column: minimise (waves of CTAs) x (planes per chunk + ring warm-up),
 // with chunks of at least 16 planes, or of any size while those would not fill the GPU once: a thread
 // walks its planes one memory latency after another (7-point constant FP64 64^3: 20.7 us a step in
@@ -134,7 +114,7 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
     if (a.plain_prefetch == 2) {
         constexpr int D = 2;
         using Col = ColumnAsync<KIND, TF, TC, true, D>;
-        auto kernel = plain_async_kernel<KIND, TF, TC, BY, D>;
+        constexpr auto kernel = plain_async_kernel<KIND, TF, TC, BY, D>;
         // Rows of more than one CTA are cut evenly, so that no CTA has its slots for a few lanes: 25-point BF16,
         // GLUP/s, 203 x 250 x 141 116 -> 120, 130 x 200 x 90 87 -> 101, 140 x 64 x 300 89 -> 106. Not rows of one CTA,
         // where a narrower one only has fewer warps: 64^3 56 -> 39-45, 33 x 500 x 100 47 -> 44.
@@ -144,21 +124,21 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
         constexpr int FULL = D * 32 * BY * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FULL);
         if (e != cudaSuccess) return e;
-        const int slots = plain_slots<KIND, TF, TC>(kernel, threads, smem);
-        const int thin = plain_slots<KIND, TF, TC>(kernel, 32 * BY, FULL);
+        const int slots = resident_ctas<kernel>(threads, smem);
+        const int thin = resident_ctas<kernel>(32 * BY, FULL);
         const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots, thin);
         const int zchunk = (L.nz + nchunks - 1) / nchunks;
         return launch_dependent(true, kernel, dim3(gx, gy, (unsigned)nchunks), dim3((unsigned)threads), smem, s, L,
                                 static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk, width);
     }
-    auto kernel = plain_sweep_kernel<KIND, TF, TC, BY, PF>;
+    constexpr auto kernel = plain_sweep_kernel<KIND, TF, TC, BY, PF>;
     // Vectors of a row per CTA. FP64 (bound by its pipe, which idle lanes hold as well): the row is cut
     // evenly and the CTA's rows follow one another in its warps, GLUP/s at 203 x 250 x 141: 7-point
     // constant 46 -> 52, 7-point variable 59 -> 63, 25-point (130 x 200 x 162) 14.6 -> 19.0. FP32 (bound
     // by HBM): a row per warp; 25-point 303 x 150 x 141 92.0 GLUP/s, cut evenly 90.8.
     const int width = sizeof(TF) == 8 ? (L.nx + (int)gx * V - 1) / ((int)gx * V) : 32;
     const int threads = (width * BY + 31) / 32 * 32;
-    const int slots = plain_slots<KIND, TF, TC>(kernel, threads);
+    const int slots = resident_ctas<kernel>(threads);
     const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots);
     const int zchunk = (L.nz + nchunks - 1) / nchunks;
     dim3 grid(gx, gy, (unsigned)nchunks);
