@@ -27,6 +27,7 @@ struct stencil_grid {
     WaveTune wtune;
     int plain_prefetch;  // plain sweep's prefetch depth (0 or 2)
     int overlap_chunks;  // overlapped sweep's z chunks (0: chosen per run)
+    bool overlap_auto;   // STENCIL_AUTO chose the overlapped sweep
     bool tune_set;
     long long launches;
     long long tile_passes;  // wavefront passes run with tile copies into shared memory
@@ -168,6 +169,7 @@ int stencil_create(stencil_t* out, int kind, int nx, int ny, int nz, int field_d
     h->scheme = STENCIL_PLAIN;
     h->tune_set = false;
     h->overlap_chunks = 0;
+    h->overlap_auto = false;
     h->launches = 0;
     h->tile_passes = 0;
     h->halo_ok = false;
@@ -362,6 +364,7 @@ int stencil_set_tuning(stencil_t h, int scheme, const stencil_tuning* tuning) {
         if (tuning && (tuning->nf < 0 || tuning->nf > h->L.nz)) return STENCIL_EINVAL;
         h->scheme = STENCIL_OVERLAP;
         h->overlap_chunks = tuning ? tuning->nf : 0;
+        h->overlap_auto = false;
         return STENCIL_OK;
     }
     if (scheme != STENCIL_BLOCKED && scheme != STENCIL_AUTO) return STENCIL_EINVAL;
@@ -377,6 +380,7 @@ int stencil_set_tuning(stencil_t h, int scheme, const stencil_tuning* tuning) {
         // measured, 64^3 to 1024^3 (overlap_impl.cuh has the figures).
         h->scheme = STENCIL_OVERLAP;
         h->overlap_chunks = 0;
+        h->overlap_auto = true;
         return STENCIL_OK;
     }
     BlockedTune t = default_tune(h);
@@ -405,17 +409,25 @@ int stencil_run(stencil_t h, int T) {
     if (!h->bound) return STENCIL_EUNBOUND;
     if (T == 0) return STENCIL_OK;
     SweepArgs a = args_of(h);
-    if (h->scheme != STENCIL_PLAIN && h->ws && !h->status_armed) {
+    int scheme = h->scheme;
+    BlockedTune tune = h->tune;
+    if (scheme == STENCIL_OVERLAP && !h->ws) {
+        // bound again without a workspace since: what AUTO selects for such a grid
+        if (!h->overlap_auto) return STENCIL_EINVAL;
+        tune = default_tune(h);
+        scheme = check_tune(h, tune) == STENCIL_OK ? STENCIL_BLOCKED : STENCIL_PLAIN;
+    }
+    if (scheme != STENCIL_PLAIN && h->ws && !h->status_armed) {
         if (cudaMemsetAsync(static_cast<int*>(h->ws) + PERSIST_WS_STATUS, 0, sizeof(int), h->stream) != cudaSuccess)
             return STENCIL_ECUDA;
         h->status_armed = true;
     }
-    if (h->scheme == STENCIL_WAVEFRONT) {
+    if (scheme == STENCIL_WAVEFRONT) {
         cudaError_t e = wave_run(a, h->field, h->parity, T, h->wtune, h->ws, GRID_WORKSPACE_BYTES, h->ctl, h->stream,
                                  &h->launches, &h->tile_passes);
         if (e == cudaErrorInvalidValue) return STENCIL_EINVAL;
         if (e != cudaSuccess) return STENCIL_ECUDA;
-    } else if (h->scheme == STENCIL_OVERLAP) {
+    } else if (scheme == STENCIL_OVERLAP) {
         cudaError_t e = overlap_run(a, h->field, h->parity, T, h->overlap_chunks, static_cast<int*>(h->ws),
                                     GRID_WORKSPACE_BYTES, h->ctl, h->stream, &h->launches);
         if (e == cudaErrorNotReady) {
@@ -431,12 +443,12 @@ int stencil_run(stencil_t h, int T) {
             }
         }
         if (e != cudaSuccess) return STENCIL_ECUDA;
-    } else if (h->scheme == STENCIL_BLOCKED) {
+    } else if (scheme == STENCIL_BLOCKED) {
         cudaError_t e = cudaErrorNotReady;
         if (h->ws) {
             // one persistent launch; if the plan for T steps does not fit one launch,
             // run the steps in two parts
-            e = blocked_run_persistent(a, h->field, h->parity, T, h->tune, h->ws, GRID_WORKSPACE_BYTES, h->ctl,
+            e = blocked_run_persistent(a, h->field, h->parity, T, tune, h->ws, GRID_WORKSPACE_BYTES, h->ctl,
                                        h->stream, &h->launches);
             if (e == cudaErrorNotReady && T > 1) {
                 int rc = stencil_run(h, T / 2);
@@ -444,7 +456,7 @@ int stencil_run(stencil_t h, int T) {
                 return stencil_run(h, T - T / 2);
             }
         }
-        if (e == cudaErrorNotReady) e = blocked_run(a, h->field, h->parity, T, h->tune, h->stream, &h->launches);
+        if (e == cudaErrorNotReady) e = blocked_run(a, h->field, h->parity, T, tune, h->stream, &h->launches);
         if (e == cudaErrorInvalidValue) return STENCIL_EINVAL;
         if (e != cudaSuccess) return STENCIL_ECUDA;
     } else {

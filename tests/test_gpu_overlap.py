@@ -72,3 +72,26 @@ def test_overlap_refuses_other_stencils():
             Stencil(kind, 20, 20, 20, dtype=dt).set_tuning("overlap")
     with pytest.raises(Exception):
         Stencil("7pt_const", 20, 20, 20).set_tuning("overlap", Tuning(6, 21, 0, 0))
+
+
+@pytest.mark.parametrize("kind,cdt", KINDS)
+def test_auto_grid_bound_again_without_a_workspace(kind, cdt):
+    """A grid that STENCIL_AUTO gave overlapped tiles and that is then bound without a workspace runs
+    what AUTO selects without one; the schedule asked for by name needs the workspace."""
+    import ctypes
+    from paper_1410_5561_gb300 import _lib as C
+    p = Problem(kind, 45, 37, 23, fdt="f32", cdt=cdt, seed=8, halo=0.5)
+    a, b, c = p.make(), p.make(), p.make()
+    a.set_tuning("plain")
+    b.set_tuning("auto")
+    c.set_tuning("overlap")
+    for s in (b, c):
+        carr = (ctypes.c_void_p * 13)(*[x.data_ptr() for x in s.coefs])
+        C.call("stencil_bind", s._h, ctypes.c_void_p(s.fields[0].data_ptr()), ctypes.c_void_p(s.fields[1].data_ptr()),
+               carr if s.ncoef else None, None)
+        s.set_field(p.torch_inputs("cuda")[0], halo=p.halo)
+    a.run(7)
+    b.run(7)
+    assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
+    with pytest.raises(C.StencilError):
+        c.run(7)
