@@ -26,20 +26,31 @@ namespace stg {
 // (upd7c_soft): 512^3 79.6 -> 120 GLUP/s, 64^3 36 -> 52, 203 x 250 x 141 49 -> 88 (cut evenly, see
 // launch_plain). GLUP/s at 512^3 by operations moved: the product 97, and one pair sum 102, two 120, three 97
 // (more integer work than the pipe saved); registers: 4 CTAs 120, 3 118, 2 110, 5 (spills) 119.
-template <int KIND, typename TF, typename TC> struct PlainCfg { static constexpr int PF = 1, MINB = 1; };
-template <typename TF> struct PlainCfg<K7C, TF, TF> { static constexpr int PF = 3, MINB = 5; };
-template <> struct PlainCfg<K7C, double, double> { static constexpr int PF = 1, MINB = 4; };
-template <> struct PlainCfg<K7V, float, float> { static constexpr int PF = 0, MINB = 3; };
-template <> struct PlainCfg<K7V, double, double> { static constexpr int PF = 0, MINB = 3; };
-template <> struct PlainCfg<K25V, float, float> { static constexpr int PF = 0, MINB = 1; };
-template <> struct PlainCfg<K25V, float, __nv_bfloat16> { static constexpr int PF = 1, MINB = 2; };
-template <> struct PlainCfg<K25V, double, double> { static constexpr int PF = 1, MINB = 2; };
+// WARP_ROWS: a row per warp that the compiler knows of. With the width of a row as an argument the constant
+// FP32 sweep, the one with the fewest operations a point, lost up to 19 % to the division and the registers that
+// hold it (GLUP/s with the argument -> without, fields set and read back: 64^3 97 -> 110, 256^3 460 -> 534, 512^3
+// 547 -> 594, 301 x 257 x 199 406 -> 488; run alone 512^3 615 -> 682, 1024^3 611 -> 700). The variable sweeps gain
+// nothing from it from 192^3 on (7-point FP32 loses 1 %) and keep the argument.
+template <int PF_, int MINB_, bool WARP_ROWS_ = false>
+struct PlainCfgOf {
+    static constexpr int PF = PF_, MINB = MINB_;
+    static constexpr bool WARP_ROWS = WARP_ROWS_;
+};
+template <int KIND, typename TF, typename TC> struct PlainCfg : PlainCfgOf<1, 1> {};
+template <> struct PlainCfg<K7C, float, float> : PlainCfgOf<3, 5, true> {};
+template <> struct PlainCfg<K7C, double, double> : PlainCfgOf<1, 4> {};
+template <> struct PlainCfg<K7V, float, float> : PlainCfgOf<0, 3> {};
+template <> struct PlainCfg<K7V, double, double> : PlainCfgOf<0, 3> {};
+template <> struct PlainCfg<K25V, float, float> : PlainCfgOf<0, 1> {};
+template <> struct PlainCfg<K25V, float, __nv_bfloat16> : PlainCfgOf<1, 2> {};
+template <> struct PlainCfg<K25V, double, double> : PlainCfgOf<1, 2> {};
 
 template <int KIND, typename TF, typename TC, int BY, int PF>
 __global__ void __launch_bounds__(32 * BY, (PlainCfg<KIND, TF, TC>::MINB))
 plain_sweep_kernel(Layout L, const TF* __restrict__ src, TF* __restrict__ dst, CoefPtrs<TC> C,
                    TF c0, TF c1, int zchunk, int width) {
     constexpr int V = 16 / sizeof(TF);
+    if (PlainCfg<KIND, TF, TC>::WARP_ROWS) width = 32;
     dependent_begin();
     const int ty = (int)threadIdx.x / width;
     const int i0 = (blockIdx.x * width + (threadIdx.x - ty * width)) * V;
