@@ -13,6 +13,7 @@
 #include "internal.h"
 #include "occupancy.h"
 #include "pdl.cuh"
+#include "plain_plan.h"
 #include "sweep_column.cuh"
 
 namespace stg {
@@ -126,21 +127,17 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
         constexpr int D = 2;
         using Col = ColumnAsync<KIND, TF, TC, true, D>;
         constexpr auto kernel = plain_async_kernel<KIND, TF, TC, BY, D>;
-        // Rows of more than one CTA are cut evenly, so that no CTA has its slots for a few lanes: 25-point BF16,
-        // GLUP/s, 203 x 250 x 141 116 -> 120, 130 x 200 x 90 87 -> 101, 140 x 64 x 300 89 -> 106. Not rows of one CTA,
-        // where a narrower one only has fewer warps: 64^3 56 -> 39-45, 33 x 500 x 100 47 -> 44.
-        const int width = gx > 1 ? (L.nx + (int)gx * V - 1) / ((int)gx * V) : 32;
-        const int threads = (width * BY + 31) / 32 * 32;
-        const size_t smem = (size_t)D * threads * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
-        constexpr int FULL = D * 32 * BY * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
+        constexpr size_t bytes = (size_t)D * (Col::SF * 16 + KindTraits<KIND>::NC * Col::CB);
+        const PrefetchShape p = prefetch_shape(L.nx, V, BY, bytes, KIND == K25V);
+        constexpr int FULL = 32 * BY * (int)bytes;
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FULL);
         if (e != cudaSuccess) return e;
-        const int slots = resident_ctas<kernel>(threads, smem);
+        const int slots = resident_ctas<kernel>(p.threads, p.smem);
         const int thin = resident_ctas<kernel>(32 * BY, FULL);
         const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots, thin);
         const int zchunk = (L.nz + nchunks - 1) / nchunks;
-        return launch_dependent(true, kernel, dim3(gx, gy, (unsigned)nchunks), dim3((unsigned)threads), smem, s, L,
-                                static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk, width);
+        return launch_dependent(true, kernel, dim3(gx, gy, (unsigned)nchunks), dim3((unsigned)p.threads), p.smem, s, L,
+                                static_cast<const TF*>(src), static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk, p.width);
     }
     constexpr auto kernel = plain_sweep_kernel<KIND, TF, TC, BY, PF>;
     // Vectors of a row per CTA. FP64 (bound by its pipe, which idle lanes hold as well): the row is cut

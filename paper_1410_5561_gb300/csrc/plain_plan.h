@@ -1,0 +1,38 @@
+// Launch plans of the plain sweep: host arithmetic, no CUDA needed.
+#pragma once
+#include <stddef.h>
+
+namespace stg {
+
+// Shared memory of an SM, and what the system reserves of it for each CTA.
+constexpr size_t SM_SHARED = 228 << 10, CTA_SHARED = 1 << 10;
+
+// Shape of a CTA of the prefetched sweep: vectors of a row, threads, shared memory.
+struct PrefetchShape {
+    int width, threads;
+    size_t smem;
+};
+// nx columns in vectors of V, rows of a CTA, shared bytes a thread's slots take; alone: one CTA an SM.
+//
+// Rows of more than one CTA (32 vectors) are cut evenly, so that no CTA has its slots for a few
+// lanes. Not rows of one CTA, where a narrower one only has fewer warps (25-point BF16, GLUP/s: 64^3 56 -> 39-45,
+// 33 x 500 x 100 47 -> 44).
+//
+// alone (the 25-point sweeps): a CTA asks for half of the SM's shared memory at least. The CTAs of
+// a cut row are small enough for two (25-point BF16: 160 or 192 threads of 560 bytes), whose slots leave
+// 49 or 13 KB of L1 to the neighbour rows that each thread copies through it and up to nine rows share. GLUP/s,
+// fields set and read back, T = 10, uncut / two CTAs / one: 176 x 256 x 200 104 / 60 / 116, 288^3 124 / 63 / 134,
+// 270 x 256 x 141 115 / 64 / 124, 130 x 200 x 90 85 / 96 / 96, 140 x 64 x 300 86 / 100 / 99, 160 x 163 x 328
+// - / 98 / 113, 203 x 250 x 141 (one either way) 112 / 116 / 116. The 7-point sweeps read one row on each side
+// and gain from two.
+inline PrefetchShape prefetch_shape(int nx, int V, int rows, size_t bytes, bool alone) {
+    PrefetchShape p;
+    const int ctas = (nx + 32 * V - 1) / (32 * V);
+    p.width = ctas > 1 ? (nx + ctas * V - 1) / (ctas * V) : 32;
+    p.threads = (p.width * rows + 31) / 32 * 32;
+    p.smem = (size_t)p.threads * bytes;
+    if (alone && ctas > 1 && p.smem < SM_SHARED / 2) p.smem = SM_SHARED / 2;
+    return p;
+}
+
+}  // namespace stg

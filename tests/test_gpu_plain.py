@@ -162,3 +162,15 @@ def test_fp64_constant_sweep_takes_every_value(shape, c0):
         assert torch.equal(torch.isnan(a), torch.isnan(b))
         ok = ~torch.isnan(a)
         assert torch.equal(a[ok].view(torch.int64), b[ok].view(torch.int64))
+
+
+@pytest.mark.parametrize("nx", [129, 141, 160, 161, 176, 192, 193, 257, 270, 288])
+def test_prefetched_25_point_rows_cut_evenly_are_bitwise_equal(nx):
+    """Rows of more than one CTA, cut evenly, at the widths where a CTA's threads change."""
+    from paper_1410_5561_gb300.stencil import Tuning
+    p = Problem("25pt_var", nx, 21, 18, fdt="f32", cdt="bf16", seed=nx, halo=0.5)
+    a, b = p.make(), p.make()
+    a.set_tuning("plain", Tuning(0, 0, 0, 0))
+    a.run(3)
+    b.run(3)
+    assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
