@@ -196,25 +196,38 @@ __global__ void fill_kernel(T* __restrict__ p, size_t n, T v) {
 // that divides both sides' addresses and the row length, four units per lane in flight; rows
 // of an odd length so move by elements. Bound by HBM, or by the launch below 128^3: a CTA per row
 // and single bytes for odd lengths took 170 us for 301 x 257 x 199 FP32, this 27 us (4.5 TB/s).
-constexpr int CPY_ROWS = 8, CPY_U = 4;
+// Few long rows are cut into segments (copy_split), so that the GPU has warps for them.
+
+// Row of this warp among ny, and the first unit of its segment.
+static __device__ __forceinline__ int copy_row(const CopySplit& c, size_t* first) {
+    const unsigned g = blockIdx.x / c.xblocks, xb = blockIdx.x - g * c.xblocks;
+    *first = (size_t)(xb * (COPY_WARPS >> c.lg) + (threadIdx.y >> c.lg)) * (size_t)c.seg;
+    return (int)((g << c.lg) + (threadIdx.y & ((1u << c.lg) - 1u)));
+}
+static dim3 copy_grid(const CopySplit& c, int ny, int nz, int arrays) {
+    const unsigned groups = (unsigned)((ny + (1 << c.lg) - 1) >> c.lg);
+    return dim3(groups * c.xblocks, (unsigned)(nz < 65535 ? nz : 65535), (unsigned)arrays);
+}
 
 template <typename U>
-__global__ void __launch_bounds__(32 * CPY_ROWS) copy_rows_kernel(const char* __restrict__ src, char* __restrict__ dst,
-                                                                  Layout L, int eb, int to_padded) {
-    const int y = (int)(blockIdx.x * CPY_ROWS + threadIdx.y);
+__global__ void __launch_bounds__(32 * COPY_WARPS) copy_rows_kernel(const char* __restrict__ src, char* __restrict__ dst,
+                                                                   Layout L, int eb, int to_padded, CopySplit c) {
+    size_t first;
+    const int y = copy_row(c, &first);
     if (y >= L.ny) return;
-    const size_t rb = (size_t)L.nx * eb, n = rb / sizeof(U);
+    const size_t rb = (size_t)L.nx * eb, all = rb / sizeof(U);
+    const size_t n = first + (size_t)c.seg < all ? first + (size_t)c.seg : all;  // the segment's end
     for (int z = (int)blockIdx.y; z < L.nz; z += (int)gridDim.y) {
         const size_t pad = L.at(0, y, z) * (size_t)eb, den = ((size_t)z * L.ny + y) * rb;
         const U* a = reinterpret_cast<const U*>(src + (to_padded ? den : pad));
         U* b = reinterpret_cast<U*>(dst + (to_padded ? pad : den));
-        for (size_t i = threadIdx.x; i < n; i += 32 * CPY_U) {
-            U v[CPY_U];
+        for (size_t i = first + threadIdx.x; i < n; i += 32 * COPY_UNITS) {
+            U v[COPY_UNITS];
 #pragma unroll
-            for (int u = 0; u < CPY_U; ++u)
+            for (int u = 0; u < COPY_UNITS; ++u)
                 if (i + 32 * u < n) v[u] = a[i + 32 * u];
 #pragma unroll
-            for (int u = 0; u < CPY_U; ++u)
+            for (int u = 0; u < COPY_UNITS; ++u)
                 if (i + 32 * u < n) b[i + 32 * u] = v[u];
         }
     }
@@ -229,16 +242,17 @@ cudaError_t copy_rows(const Layout& L, int eb, const void* src, void* dst, bool 
     if (L.nx == 0 || L.ny == 0 || L.nz == 0) return cudaSuccess;
     const uintptr_t bits = (uintptr_t)src | (uintptr_t)dst | ((uintptr_t)L.nx * eb) | ((uintptr_t)L.xo * eb) |
                            ((uintptr_t)L.px * eb);
-    const dim3 grid((unsigned)((L.ny + CPY_ROWS - 1) / CPY_ROWS), (unsigned)(L.nz < 65535 ? L.nz : 65535));
-    const dim3 block(32, CPY_ROWS);
+    const int unit = copy_unit(bits, eb);
+    const CopySplit c = copy_split(L.ny, (long long)L.ny * L.nz, (long long)L.nx * eb / unit);
+    const dim3 grid = copy_grid(c, L.ny, L.nz, 1), block(32, COPY_WARPS);
     const char* a = static_cast<const char*>(src);
     char* b = static_cast<char*>(dst);
-    switch (copy_unit(bits, eb)) {
-        case 16: copy_rows_kernel<uint4><<<grid, block, 0, s>>>(a, b, L, eb, to_padded); break;
-        case 8: copy_rows_kernel<uint2><<<grid, block, 0, s>>>(a, b, L, eb, to_padded); break;
-        case 4: copy_rows_kernel<unsigned><<<grid, block, 0, s>>>(a, b, L, eb, to_padded); break;
-        case 2: copy_rows_kernel<unsigned short><<<grid, block, 0, s>>>(a, b, L, eb, to_padded); break;
-        default: copy_rows_kernel<unsigned char><<<grid, block, 0, s>>>(a, b, L, eb, to_padded); break;
+    switch (unit) {
+        case 16: copy_rows_kernel<uint4><<<grid, block, 0, s>>>(a, b, L, eb, to_padded, c); break;
+        case 8: copy_rows_kernel<uint2><<<grid, block, 0, s>>>(a, b, L, eb, to_padded, c); break;
+        case 4: copy_rows_kernel<unsigned><<<grid, block, 0, s>>>(a, b, L, eb, to_padded, c); break;
+        case 2: copy_rows_kernel<unsigned short><<<grid, block, 0, s>>>(a, b, L, eb, to_padded, c); break;
+        default: copy_rows_kernel<unsigned char><<<grid, block, 0, s>>>(a, b, L, eb, to_padded, c); break;
     }
     return cudaGetLastError();
 }
@@ -252,29 +266,32 @@ struct PackArgs {
 };
 
 template <typename U>
-__global__ void __launch_bounds__(32 * CPY_ROWS) pack_rows_kernel(const __grid_constant__ PackArgs P, Layout L, int eb) {
-    const int r = (int)(blockIdx.x * CPY_ROWS + threadIdx.y);
+__global__ void __launch_bounds__(32 * COPY_WARPS) pack_rows_kernel(const __grid_constant__ PackArgs P, Layout L, int eb,
+                                                                   CopySplit c) {
+    size_t first;
+    const int r = copy_row(c, &first);
     if (r >= L.py) return;
     const char* const src = P.src[blockIdx.z];
     char* const dst = P.dst[blockIdx.z];
     const long long lo = (long long)L.xo * eb / (int)sizeof(U), n = (long long)L.nx * eb / (int)sizeof(U);
-    const long long np = (long long)L.px * eb / (int)sizeof(U);
+    const long long all = (long long)L.px * eb / (int)sizeof(U);
+    const long long np = (long long)first + c.seg < all ? (long long)first + c.seg : all;  // the segment's end
     const int y = r - L.R;
     for (int q = (int)blockIdx.y; q < L.pz; q += (int)gridDim.y) {
         const int z = q - L.R;
         const bool in = y >= 0 && y < L.ny && z >= 0 && z < L.nz;
         const U* a = reinterpret_cast<const U*>(src + (in ? ((size_t)z * L.ny + y) * ((size_t)L.nx * eb) : 0));
         U* b = reinterpret_cast<U*>(dst + ((size_t)q * L.py + r) * ((size_t)L.px * eb));
-        for (long long i = threadIdx.x; i < np; i += 32 * CPY_U) {
-            U v[CPY_U];
+        for (long long i = (long long)first + threadIdx.x; i < np; i += 32 * COPY_UNITS) {
+            U v[COPY_UNITS];
 #pragma unroll
-            for (int u = 0; u < CPY_U; ++u) {
+            for (int u = 0; u < COPY_UNITS; ++u) {
                 const long long x = i + 32 * u - lo;
                 v[u] = U{};
                 if (in && x >= 0 && x < n) v[u] = a[x];
             }
 #pragma unroll
-            for (int u = 0; u < CPY_U; ++u)
+            for (int u = 0; u < COPY_UNITS; ++u)
                 if (i + 32 * u < np) b[i + 32 * u] = v[u];
         }
     }
@@ -288,14 +305,15 @@ cudaError_t pack_rows(const Layout& L, int eb, const void* const* src, void* con
         P.dst[m] = static_cast<char*>(dst[m]);
         bits |= (uintptr_t)src[m] | (uintptr_t)dst[m];
     }
-    const dim3 grid((unsigned)((L.py + CPY_ROWS - 1) / CPY_ROWS), (unsigned)(L.pz < 65535 ? L.pz : 65535), (unsigned)n);
-    const dim3 block(32, CPY_ROWS);
-    switch (copy_unit(bits, eb)) {
-        case 16: pack_rows_kernel<uint4><<<grid, block, 0, s>>>(P, L, eb); break;
-        case 8: pack_rows_kernel<uint2><<<grid, block, 0, s>>>(P, L, eb); break;
-        case 4: pack_rows_kernel<unsigned><<<grid, block, 0, s>>>(P, L, eb); break;
-        case 2: pack_rows_kernel<unsigned short><<<grid, block, 0, s>>>(P, L, eb); break;
-        default: pack_rows_kernel<unsigned char><<<grid, block, 0, s>>>(P, L, eb); break;
+    const int unit = copy_unit(bits, eb);
+    const CopySplit c = copy_split(L.py, (long long)L.py * L.pz * n, (long long)L.px * eb / unit);
+    const dim3 grid = copy_grid(c, L.py, L.pz, n), block(32, COPY_WARPS);
+    switch (unit) {
+        case 16: pack_rows_kernel<uint4><<<grid, block, 0, s>>>(P, L, eb, c); break;
+        case 8: pack_rows_kernel<uint2><<<grid, block, 0, s>>>(P, L, eb, c); break;
+        case 4: pack_rows_kernel<unsigned><<<grid, block, 0, s>>>(P, L, eb, c); break;
+        case 2: pack_rows_kernel<unsigned short><<<grid, block, 0, s>>>(P, L, eb, c); break;
+        default: pack_rows_kernel<unsigned char><<<grid, block, 0, s>>>(P, L, eb, c); break;
     }
     return cudaGetLastError();
 }

@@ -35,4 +35,29 @@ inline PrefetchShape prefetch_shape(int nx, int V, int rows, size_t bytes, bool 
     return p;
 }
 
+// How the interior copies cut their rows: a CTA of COPY_WARPS warps has 1 << lg neighbouring rows and
+// COPY_WARPS >> lg segments of `seg` units of each; the CTAs of a group of rows (xblocks) follow one
+// another. Rows are cut as far as there would be fewer than COPY_WANT warps (64 an SM), but not below one pass
+// of a warp (32 lanes of COPY_UNITS units): a warp that moves a whole long row has 2 KB under way, and few such rows
+// leave the GPU idle. A field set and read back and its sweep, FP32, T = 4, whole rows -> cut: 1000000 x 1 x 1 1099
+// -> 43 us, 100000 x 8 x 4 193 -> 37, 20000 x 3 x 5 37 -> 26. Grids of 9728 rows or more are copied by whole rows.
+constexpr int COPY_WARPS = 8, COPY_UNITS = 4;
+constexpr long long COPY_WANT = 152 * 64;
+
+struct CopySplit {
+    int lg;
+    unsigned xblocks;
+    long long seg;
+};
+// ny rows a plane, rows in all, units a row.
+inline CopySplit copy_split(int ny, long long rows, long long units) {
+    CopySplit c;
+    c.lg = ny >= 8 ? 3 : ny >= 4 ? 2 : ny >= 2 ? 1 : 0;
+    const long long want = (COPY_WANT + rows - 1) / rows, pass = 32 * COPY_UNITS;
+    c.seg = ((units + want - 1) / want + pass - 1) / pass * pass;
+    const long long segs = (units + c.seg - 1) / c.seg, per = COPY_WARPS >> c.lg;
+    c.xblocks = (unsigned)((segs + per - 1) / per);
+    return c;
+}
+
 }  // namespace stg

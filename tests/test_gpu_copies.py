@@ -35,3 +35,26 @@ def test_coefficients_and_field_land_in_the_padded_arrays(nx, dt, cdt, off):
     assert torch.equal(s.get_field(out), u)
     s.current.fill_(0.5)
     assert bool((s.fields[0] == 0.5).all())
+
+
+@pytest.mark.parametrize("shape", [(70001, 1, 1), (40000, 2, 1), (9001, 5, 3), (130004, 8, 1)])
+@pytest.mark.parametrize("dt,cdt", [("float32", "float32"), ("float32", "bfloat16"), ("float64", "float64")])
+def test_long_rows_are_copied_in_segments(shape, dt, cdt):
+    import torch
+    from paper_1410_5561_gb300.stencil import Stencil
+    nx, ny, nz = shape
+    s = Stencil("7pt_var", nx, ny, nz, dtype=getattr(torch, dt), coef_dtype=getattr(torch, cdt))
+    g = torch.Generator(device="cuda").manual_seed(nx)
+    arrs = [torch.rand(nz, ny, nx, generator=g, device="cuda").to(s.coef_dtype) for _ in range(7)]
+    u = torch.rand(nz, ny, nx, generator=g, device="cuda", dtype=s.dtype)
+    for c in s.coefs:
+        c.fill_(9.0)
+    s.set_coeffs(arrays=arrs)
+    s.set_field(u, halo=0.5)
+    for m in range(7):
+        assert torch.equal(s.coef_interior(m), arrs[m])
+        s.coef_interior(m).zero_()
+        assert not bool(s.coefs[m].any())
+    assert torch.equal(s.get_field(), u)
+    s.current.fill_(0.5)
+    assert bool((s.fields[0] == 0.5).all())

@@ -14,6 +14,13 @@ extern "C" long prefetch(int nx, int V, int rows, long bytes, int alone, int* th
     *smem = (long)p.smem;
     return p.width;
 }
+extern "C" int split(int ny, long rows, long units, long* xblocks, long* seg) {
+    const stg::CopySplit c = stg::copy_split(ny, rows, units);
+    *xblocks = c.xblocks;
+    *seg = (long)c.seg;
+    return c.lg;
+}
+extern "C" long want() { return (long)stg::COPY_WANT; }
 """
 SM_SHARED, CTA_SHARED, CTA_MOST = 228 << 10, 1 << 10, 227 << 10
 
@@ -39,3 +46,23 @@ def test_prefetched_25_point_rows_of_several_ctas_run_one_an_sm(lib, V, bytes_):
         assert t.value * bytes_ <= m.value <= max(256 * bytes_, SM_SHARED // 2) <= CTA_MOST
         if ctas > 1:
             assert 2 * (m.value + CTA_SHARED) > SM_SHARED, nx
+
+
+@pytest.mark.parametrize("ny", [1, 2, 3, 4, 7, 8, 9, 33, 4000])
+@pytest.mark.parametrize("nz", [1, 2, 5, 3000])
+def test_copies_cover_every_row_once_with_warps_for_the_gpu(lib, ny, nz):
+    """Segments of a row follow one another and end with it, rows of a CTA likewise; few rows give as
+    many warps as the GPU wants, or as there are passes of a warp; many rows are not cut."""
+    lib.want.restype = ctypes.c_long
+    for units in (1, 2, 31, 127, 128, 129, 1000, 4097, 20000, 250000, 1 << 21):
+        xb, seg = ctypes.c_long(), ctypes.c_long()
+        lg = lib.split(ny, ctypes.c_long(ny * nz), ctypes.c_long(units), ctypes.byref(xb), ctypes.byref(seg))
+        per, seg, xb = 8 >> lg, seg.value, xb.value
+        assert 1 << lg <= max(ny, 1) and (1 << lg) * per == 8
+        segs = -(-units // seg)
+        assert (xb - 1) * per < segs <= xb * per and -(-ny // (1 << lg)) * xb < 2 ** 31
+        passes = -(-units // 128)
+        assert seg % 128 == 0
+        assert 2 * ny * nz * segs >= min(lib.want(), ny * nz * passes)
+        if ny * nz >= lib.want():
+            assert segs == 1
