@@ -145,7 +145,11 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
     // constant 46 -> 52, 7-point variable 59 -> 63, 25-point (130 x 200 x 162) 14.6 -> 19.0. FP32 (bound
     // by HBM): a row per warp; 25-point 303 x 150 x 141 92.0 GLUP/s, cut evenly 90.8.
     const int width = sizeof(TF) == 8 ? (L.nx + (int)gx * V - 1) / ((int)gx * V) : 32;
-    const int threads = (width * BY + 31) / 32 * 32;
+    // FP64 grids of fewer than BY rows have no threads for the others, so that more CTAs fit: 7-point constant 4096 x 1
+    // x 4096, about 240 us a step, with 7 of 8 warps idle 750 (and 380 before it formed some operations on the
+    // integer pipes, which one warp a scheduler does not hide).
+    const int rows = sizeof(TF) == 8 && L.ny < BY ? L.ny : BY;
+    const int threads = (width * rows + 31) / 32 * 32;
     const int slots = resident_ctas<kernel>(threads);
     const int nchunks = plain_chunks((long long)gx * gy, L.nz, KindTraits<KIND>::R, slots);
     const int zchunk = (L.nz + nchunks - 1) / nchunks;

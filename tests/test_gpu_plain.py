@@ -174,3 +174,17 @@ def test_prefetched_25_point_rows_cut_evenly_are_bitwise_equal(nx):
     a.run(3)
     b.run(3)
     assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
+
+
+@pytest.mark.parametrize("kind", ["7pt_const", "7pt_var", "25pt_var"])
+@pytest.mark.parametrize("ny", [1, 2, 3, 7, 8, 9])
+@pytest.mark.parametrize("nx", [5, 64, 131])
+def test_fp64_sweep_of_few_rows_is_bitwise_equal(kind, ny, nx):
+    """FP64 CTAs of fewer rows than usual against the prefetched form, which has them all."""
+    from paper_1410_5561_gb300.stencil import Tuning
+    p = Problem(kind, nx, ny, 23, fdt="f64", seed=nx + ny, halo=0.375)
+    a, b = p.make(), p.make()
+    a.run(3)
+    b.set_tuning("plain", Tuning(0, 2, 0, 0))
+    b.run(3)
+    assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
