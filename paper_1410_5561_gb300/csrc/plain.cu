@@ -155,10 +155,8 @@ static cudaError_t launch_plain(const SweepArgs& a, const void* src, void* dst, 
     const int zchunk = (L.nz + nchunks - 1) / nchunks;
     dim3 grid(gx, gy, (unsigned)nchunks);
     // Set up beside the step before it (pdl.cuh), 64^3, us per step: 7-point constant FP64 20.7 -> 7.4, FP32
-    // 9.5 -> 2.8 (thinner chunks included), at 256^3 33.0 -> 31.0. Not FP64 sweeps of several waves: they
-    // are bound by the FP64 units, which the uneven second wave then loads unevenly (1 % slower at
-    // 203 x 250 x 141).
-    const bool early = sizeof(TF) == 4 || (long long)gx * gy * nchunks <= slots;
+    // 9.5 -> 2.8 (thinner chunks included), at 256^3 33.0 -> 31.0. Not every FP64 sweep (early_fp64).
+    const bool early = sizeof(TF) == 4 || early_fp64((long long)gx * gy * nchunks, slots, zchunk);
     return launch_dependent(early, kernel, grid, dim3((unsigned)threads), 0, s, L, static_cast<const TF*>(src),
                             static_cast<TF*>(dst), C, (TF)a.c0, (TF)a.c1, zchunk, width);
 }

@@ -35,6 +35,18 @@ inline PrefetchShape prefetch_shape(int nx, int V, int rows, size_t bytes, bool 
     return p;
 }
 
+// Whether an FP64 step of `ctas` CTAs, of which the GPU holds `slots`, with walks of `planes` planes is set up
+// beside the step before it. FP64 sweeps are bound by the FP64 units, which CTAs that are set up early load
+// unevenly: those of a second wave (1 % slower at 203 x 250 x 141), and those that find free slots
+// beside a step that does not fill the GPU, on the SMs that have fewest of its CTAs, for the
+// whole of a long walk. Speed with / without, fill of the slots and planes a walk: 7-point variable 469 x 230 x 29 0.76
+// (0.51, 29), constant 600 x 300 x 30 0.82 (0.62, 30), 253 x 429 x 32 0.85 (0.71, 16), 328 x 461 x 19 0.93 (0.57, 19),
+// 393 x 183 x 40 0.98 (0.79, 14); 186 x 332 x 83 0.99 (0.83, 21), 500 x 500 x 28 1.02 (0.83, 28), 81 x 99 x 44 1.15
+// (0.75, 2), 64^3 1.24 (0.84, 1).
+inline bool early_fp64(long long ctas, int slots, int planes) {
+    return ctas <= slots && (5 * ctas >= 4LL * slots || planes < 12);
+}
+
 // How the interior copies cut their rows: a CTA of COPY_WARPS warps has 1 << lg neighbouring rows and
 // COPY_WARPS >> lg segments of `seg` units of each; the CTAs of a group of rows (xblocks) follow one
 // another. Rows are cut as far as there would be fewer than COPY_WANT warps (64 an SM), but not below one pass

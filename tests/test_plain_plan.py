@@ -20,6 +20,7 @@ extern "C" int split(int ny, long rows, long units, long* xblocks, long* seg) {
     *seg = (long)c.seg;
     return c.lg;
 }
+extern "C" int early(long ctas, int slots, int planes) { return stg::early_fp64(ctas, slots, planes) ? 1 : 0; }
 extern "C" long want() { return (long)stg::COPY_WANT; }
 """
 SM_SHARED, CTA_SHARED, CTA_MOST = 228 << 10, 1 << 10, 227 << 10
@@ -66,3 +67,12 @@ def test_copies_cover_every_row_once_with_warps_for_the_gpu(lib, ny, nz):
         assert 2 * ny * nz * segs >= min(lib.want(), ny * nz * passes)
         if ny * nz >= lib.want():
             assert segs == 1
+
+
+@pytest.mark.parametrize("ctas,slots,planes,want", [
+    (232, 456, 29, 0), (375, 608, 30, 0), (432, 608, 16, 0), (483, 608, 14, 0),  # measured 0.76 to 0.98 when early
+    (608, 608, 23, 1), (505, 608, 21, 1), (570, 760, 2, 1), (513, 608, 1, 1), (41, 608, 1, 1),
+    (609, 608, 1, 0), (1200, 608, 30, 0),  # several waves
+])
+def test_fp64_steps_set_up_early(lib, ctas, slots, planes, want):
+    assert lib.early(ctypes.c_long(ctas), slots, planes) == want
