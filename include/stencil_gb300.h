@@ -170,8 +170,9 @@ int stencil_set_field(stencil_t h, const void* src, double halo_value, int where
  * column of tiles, 0 or NULL: chosen from the grid and the GPU; other fields ignored;
  * bit-identical to the plain sweep), or
  * STENCIL_AUTO (plain for FP64 fields and the 25-point stencil, where the plain sweep
- * measured faster on GB300; overlapped tiles for the 7-point stencils in FP32; without a
- * workspace the default blocked tuning when it fits, else plain).
+ * measured faster on GB300; overlapped tiles for the 7-point stencils in FP32, except that thin
+ * or small grids of more than 1808 points a row and runs of fewer than three steps take plain
+ * steps; without a workspace the default blocked tuning when it fits, else plain).
  * Returns STENCIL_ENOSMEM / STENCIL_EINVAL for an infeasible blocked tuning. */
 int stencil_set_tuning(stencil_t h, int scheme, const stencil_tuning* tuning);
 

@@ -113,6 +113,29 @@ static int check_tune(const stencil_grid* h, const BlockedTune& t) {
     return STENCIL_OK;
 }
 
+// Whether AUTO gives a 7-point FP32 grid overlapped tiles; else the plain sweep. Rows too long for the diamonds
+// (16 x tiles: more than 1808 points) had the plain sweep before there were overlapped tiles, and have it where
+// those have too little to share over three steps: up to two planes (GLUP/s with fields set and read back, T = 30,
+// overlapped / plain: 7-point constant 2000 x 2000 x 1 222 / 424, FP32 coefficients 69 / 137, BF16 89 / 218; two
+// planes 391 / 518, 118 / 155, 153 / 244; four 619 / 548, 187 / 168, 242 / 256), fewer than 2^20 points (2000 x 31
+// x 6: 81 / 143, 83 / 120, 73 / 142), and, but for FP32 coefficients, which HBM bounds either way, rows
+// that fill few warps of a tile (2000 x 1 x 2000: 99 / 133, 71 / 42, 66 / 71; 5000 x 3 x 124 and 5000 x 6 x 201
+// 0.46 and 0.81 of the plain sweep, BF16 0.77 and 0.89; 2000 x 4 x 2000 1.18 and 1.27).
+//
+// On shorter rows AUTO keeps to one launch a run, also on small grids, where the plain sweep's steps
+// have become the faster ones (T = 100 alone, overlapped / plain: 7-point constant 64^3 67 / 125, 96^3 220 / 284,
+// 112^3 337 / 334, 128^3 488 / 470, 160^3 624 / 466; FP32 coefficients 64 / 79, 176 / 191, 240 / 210, 312 / 165,
+// 252 / 152; BF16 57 / 95, 175 / 244, 263 / 297, 341 / 275, 327 / 250).
+static bool auto_overlap(const stencil_grid* h) {
+    const Layout& L = h->L;
+    if (check_tune(h, default_tune(h)) == STENCIL_OK) return true;
+    const long long points = (long long)L.nx * L.ny * L.nz;
+    const bool bf16 = h->cdt == STENCIL_BF16;
+    if (L.nz <= (bf16 ? 4 : 2) || points < (1 << 20)) return false;
+    if (h->kind == STENCIL_7PT_VAR && !bf16) return true;
+    return !(L.ny <= 2 || (L.ny < 8 && points < (1 << 23)));
+}
+
 namespace stg {
 int grid_batch_view(const stencil_grid* h, SweepArgs* a, void** f0, void** f1, int* parity) {
     if (!h) return STENCIL_EINVAL;
@@ -376,9 +399,9 @@ int stencil_set_tuning(stencil_t h, int scheme, const stencil_tuning* tuning) {
         return STENCIL_OK;
     }
     if (scheme == STENCIL_AUTO && overlap_ok(args_of(h)) && h->ws) {
-        // The 7-point stencils in FP32: faster than the plain sweep and the diamonds at every size
-        // measured, 64^3 to 1024^3 (overlap_impl.cuh has the figures).
-        h->scheme = STENCIL_OVERLAP;
+        // The 7-point stencils in FP32: overlapped tiles. They are faster than the diamonds on every grid
+        // measured, and than the plain sweep from about 112^3 on (auto_overlap has the figures).
+        h->scheme = auto_overlap(h) ? STENCIL_OVERLAP : STENCIL_PLAIN;
         h->overlap_chunks = 0;
         h->overlap_auto = true;
         return STENCIL_OK;
@@ -416,6 +439,14 @@ int stencil_run(stencil_t h, int T) {
         if (!h->overlap_auto) return STENCIL_EINVAL;
         tune = default_tune(h);
         scheme = check_tune(h, tune) == STENCIL_OK ? STENCIL_BLOCKED : STENCIL_PLAIN;
+    }
+    if (scheme == STENCIL_OVERLAP && h->overlap_auto && T < 3 &&
+        !(h->kind == STENCIL_7PT_CONST && (long long)h->L.nx * h->L.ny * h->L.nz >= (1 << 28))) {
+        // No pass of three steps: nothing that the tiles' overlap is paid back by. Time of a step, plain over
+        // overlapped, with fields set and read back: 7-point constant 128^3 0.67, 256^3 0.76, 512^3 0.99
+        // (768^3 1.02), FP32 coefficients 0.64, 0.84, 0.91, BF16 0.55, 0.75, 0.90; rows of 1500 points and
+        // more (plain before there were overlapped tiles) 0.27 to 0.99.
+        scheme = STENCIL_PLAIN;
     }
     if (scheme != STENCIL_PLAIN && h->ws && !h->status_armed) {
         if (cudaMemsetAsync(static_cast<int*>(h->ws) + PERSIST_WS_STATUS, 0, sizeof(int), h->stream) != cudaSuccess)

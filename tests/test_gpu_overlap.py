@@ -95,3 +95,23 @@ def test_auto_grid_bound_again_without_a_workspace(kind, cdt):
     assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
     with pytest.raises(C.StencilError):
         c.run(7)
+
+
+@pytest.mark.parametrize("kind,cdt", KINDS)
+@pytest.mark.parametrize("shape,T,launches", [
+    ((70, 23, 19), 9, 1), ((70, 23, 19), 2, 2), ((70, 23, 19), 1, 1),   # no pass of three steps: plain steps
+    ((1808, 30, 2), 3, 1), ((1809, 300, 2), 3, 3), ((1809, 20, 20), 3, 3), ((2000, 60, 12), 3, 1),
+])
+def test_auto_between_overlapped_tiles_and_plain_steps(kind, cdt, shape, T, launches):
+    """AUTO runs plain steps where the overlapped tiles have nothing to share: fewer than three steps, and thin
+    or small grids of long rows. The same bits either way."""
+    p = Problem(kind, *shape, fdt="f32", cdt=cdt, seed=31, halo=0.25)
+    a, b = p.make(), p.make()
+    a.set_tuning("plain")
+    b.set_tuning("auto")
+    a.run(T)
+    n0 = b.launches
+    b.run(T)
+    assert b.launches == n0 + launches
+    assert a.parity == b.parity
+    assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
