@@ -139,3 +139,60 @@ def test_batch_autotuner_choice_is_feasible_and_exact():
         got = g.get_field().cpu().numpy()
         _check_oracle(p, T, got)
         assert np.array_equal(got, _plain_result(p, T))
+
+
+# stencils and types whose batches run the diamonds
+DIAMONDS = [("7pt_const", "f64", None, (4, 1, 8)), ("7pt_var", "f64", None, (4, 2, 8)), ("25pt_var", "f32", None, (8, 1, 8))]
+
+
+@pytest.mark.parametrize("kind,fdt,cdt,tn", DIAMONDS)
+def test_diamond_batch_graph_replay(kind, fdt, cdt, tn):
+    import torch
+    from paper_1410_5561_gb300.batch import Batch
+    from paper_1410_5561_gb300.stencil import Tuning
+    probs = _problems(kind, fdt, cdt)
+    grids = [p.make() for p, _ in probs]
+    b = Batch(grids, [T for _, T in probs], Tuning(*tn, 0))
+    b.launch()
+    torch.cuda.synchronize()
+    graph = b.capture()
+    graph.replay()
+    graph.replay()
+    torch.cuda.synchronize()
+    b.sync_parity()
+    assert b.status() == 0
+    for (p, T), g in zip(probs, grids):
+        assert np.array_equal(g.get_field().cpu().numpy(), _plain_result(p, 3 * T))
+
+
+@pytest.mark.parametrize("kind,fdt,cdt,tn", DIAMONDS)
+def test_diamond_batch_timeout_is_reported_not_hung(kind, fdt, cdt, tn):
+    import torch
+    from paper_1410_5561_gb300._lib import STATUS
+    from paper_1410_5561_gb300.batch import Batch
+    from paper_1410_5561_gb300.stencil import Tuning
+    probs = _problems(kind, fdt, cdt)
+    grids = [p.make() for p, _ in probs]
+    b = Batch(grids, [T for _, T in probs], Tuning(*tn, 0))
+    b.set_wait_limit(2000)
+    b.inject_stall(b.items // 2)
+    b.launch()
+    torch.cuda.synchronize()
+    assert STATUS[b.status()] == "STENCIL_ETIMEOUT"
+
+
+def test_diamond_batch_autotuner_choice_is_feasible_and_exact():
+    from paper_1410_5561_gb300 import tuner
+    from paper_1410_5561_gb300.batch import Batch
+    from paper_1410_5561_gb300.stencil import Tuning
+    probs = _problems("7pt_var", "f64")
+    Ts = [T for _, T in probs]
+    cands = [Tuning(4, 1, 8, 0), Tuning(4, 2, 8, 0), Tuning(64, 8, 8, 0)]
+    tn, table = tuner.tune_batch([p.make() for p, _ in probs], Ts, cands, reps=1)
+    assert tn in cands[:2] and [c for c, _ in table] == cands[:2]
+    fresh = [p.make() for p, _ in probs]
+    b = Batch(fresh, Ts, tn)
+    b.launch()
+    assert b.status() == 0
+    for (p, T), g in zip(probs, fresh):
+        assert np.array_equal(g.get_field().cpu().numpy(), _plain_result(p, T))

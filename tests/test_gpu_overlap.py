@@ -115,3 +115,47 @@ def test_auto_between_overlapped_tiles_and_plain_steps(kind, cdt, shape, T, laun
     assert b.launches == n0 + launches
     assert a.parity == b.parity
     assert np.array_equal(a.get_field().cpu().numpy(), b.get_field().cpu().numpy())
+
+
+@pytest.mark.parametrize("kind,cdt", KINDS)
+def test_overlap_timeout_is_reported_not_hung(kind, cdt):
+    """A tile made to wait on a flag that no tile sets, with a short wait limit, ends the launch with the
+    status word set; a new field clears it and the next run is exact."""
+    from paper_1410_5561_gb300._lib import STATUS, StencilError
+    p = Problem(kind, 140, 64, 24, fdt="f32", cdt=cdt, seed=9)
+    a, s = p.make(), p.make()
+    a.set_tuning("plain")
+    a.run(13)
+    s.set_tuning("overlap")
+    s.set_wait_limit(2000)
+    s.inject_stall(5)
+    s.run(13)
+    assert STATUS[s.status()] == "STENCIL_ETIMEOUT"
+    with pytest.raises(StencilError):
+        s.sync()
+    s.inject_stall(-1)
+    s.set_wait_limit(1 << 24)
+    s.set_field(p.torch_inputs("cuda")[0], halo=p.halo)
+    s.run(13)
+    assert s.status() == 0
+    assert np.array_equal(s.get_field().cpu().numpy(), a.get_field().cpu().numpy())
+
+
+def test_overlap_with_more_tiles_than_counters():
+    """Chunks of four planes of a grid of 2^24 planes are more tiles than the workspace has counters for: the
+    run is cut in two and takes plain steps."""
+    import torch
+    from paper_1410_5561_gb300.stencil import Stencil, Tuning
+    nz = 1 << 24
+    s = Stencil("7pt_const", 1, 1, nz)
+    s.set_coeffs(scalars=(0.4, 0.1))
+    u = torch.rand(nz, 1, 1, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    s.set_field(u, halo=0.25)
+    s.run(7)
+    ref = s.get_field().clone()
+    s.set_field(u, halo=0.25)
+    s.set_tuning("overlap", Tuning(6, nz, 0, 0))
+    n0 = s.launches
+    s.run(7)
+    assert s.launches == n0 + 7 and s.parity == 1
+    assert torch.equal(s.get_field(), ref)

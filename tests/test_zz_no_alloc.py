@@ -79,3 +79,30 @@ def test_noalloc_batch_rejects_a_plan_beyond_its_scratch():
     assert status.value == -99
     for g, b in zip(grids, before):
         assert g.parity == 0 and np.array_equal(g.get_field().cpu().numpy(), b)
+
+
+def test_noalloc_batch_takes_the_diamonds_where_overlapped_tiles_do_not_fit():
+    """9000 steps of a 160 x 160 x 16 grid are more overlapped tiles than the scratch holds; the
+    diamonds of the same batch fit, so the call runs, on them."""
+    import torch
+    from paper_1410_5561_gb300 import _lib as C
+    from paper_1410_5561_gb300.stencil import Tuning
+    from tests._util import Problem
+
+    p = Problem("7pt_var", 160, 160, 16, fdt="f32", seed=77, halo=0.25)
+    a, s = p.make(), p.make()
+    T = 9000
+    hs, ts, t = _handles([s]), (ctypes.c_int * 1)(T), Tuning(8, 1, 16, 0).c()
+    b = ctypes.c_void_p()
+    C.call("stencil_batch_create", ctypes.byref(b), hs, ts, 1, ctypes.byref(t))
+    try:
+        assert int(C.lib().stencil_batch_workspace_bytes(b)) > (4 << 20)
+    finally:
+        C.lib().stencil_batch_destroy(b)
+    status = ctypes.c_int(-99)
+    C.call("stencil_batch_run_noalloc", hs, ts, 1, ctypes.byref(t),
+           ctypes.c_void_p(torch.cuda.current_stream().cuda_stream), ctypes.byref(status))
+    assert status.value == 0
+    a.set_tuning("plain")
+    a.run(T)
+    assert np.array_equal(a.get_field().cpu().numpy(), s.get_field().cpu().numpy())
