@@ -126,7 +126,11 @@ def candidates(s: Stencil, nfs=(1, 2), warps=(8, 16), max_dw=None) -> list[Tunin
 # for the 7-point variable stencil with FP32 coefficients, whose two frontlines wait on their
 # coefficient loads one after the other: there one frontline is 6 % cheaper (215 vs 201 GLUP/s
 # at 384^3, T = 50).
+# The overlapped tiles stream one pass of three steps at 0.75 of the copy rate (7-point constant 1024^3,
+# 7-point variable FP32 384^3; BF16 coefficients 0.5, bound by their widening).
 PLAIN_STREAM = 0.83
+OVERLAP_STREAM = {"f32": 0.75, "bf16": 0.5}
+OVERLAP_STEPS = 3
 BLOCKED_STREAM = 0.42
 SPILL = {1: 1.0, 2: 3.0, 4: 7.0}
 NF_COST = {1: 1.23, 2: 1.0}
@@ -149,7 +153,8 @@ def predict(s: Stencil, T: int, scheme: str, t: Tuning | None = None, hbm_gbs: f
     streaming rate and the floating-point instructions at ``fp_peak`` FLOP/s (FP64 sweeps are
     bound by GB300's FP64 units); blocked: Eq. 5's code balance at the diamond kernel's
     streaming rate, divided by the useful share of computed x columns, times the register
-    (items per warp) and frontline factors; wavefront: the plain sweep's rate, since every time
+    (items per warp) and frontline factors; overlap: the plain sweep's bytes once per three steps
+    and once per step of the remainder, at the overlapped tiles' streaming rate; wavefront: the plain sweep's rate, since every time
     level keeps pace with level 0, which has h^-1 of the CTAs (measured: the schedule cuts HBM
     bytes but not time)."""
     kind = _KIND_NAME[s.kind]
@@ -164,6 +169,9 @@ def predict(s: Stencil, T: int, scheme: str, t: Tuning | None = None, hbm_gbs: f
     if scheme in ("plain", "wavefront"):
         b = model.bytes_per_lup(kind, fdt, cdt, "plain")
         return max(lups * b / (PLAIN_STREAM * hbm_gbs * 1e9), alu)
+    if scheme == "overlap":
+        b = model.bytes_per_lup(kind, fdt, cdt, "plain") * (T // OVERLAP_STEPS + T % OVERLAP_STEPS) / max(T, 1)
+        return max(lups * b / (OVERLAP_STREAM[cdt] * hbm_gbs * 1e9), alu)
     b = model.bytes_per_lup(kind, fdt, cdt, "blocked", t.dw)
     lt = t.dw // r - 1
     ov = -(-r * (lt - 1) // v) if lt > 1 else 0
@@ -196,7 +204,9 @@ def autotune(s: Stencil, T: int, reps: int = 2, max_candidates: int = 10, includ
     """Pick the fastest schedule for ``T`` steps of grid ``s``, guided by ``predict``.
 
     Candidates: the plain sweep, the first ``max_candidates`` blocked tunings of
-    ``candidates`` (capacity-pruned) and, if asked, the library's default wavefront tuning.
+    ``candidates`` (capacity-pruned) and, if ``schemes`` names them, the library's default
+    wavefront tuning and, for the 7-point stencils in FP32, the overlapped tiles that
+    ``set_tuning("auto")`` gives such grids (the fastest of all on large ones: name "overlap" there).
     Each is predicted; the best prediction is timed first and fixes the model's absolute
     scale; candidates predicted more than 1.5x slower than the best are dropped; at most
     ``max_timed`` are timed, in predicted order. Returns (scheme, tuning or None, table), the
@@ -215,6 +225,8 @@ def autotune(s: Stencil, T: int, reps: int = 2, max_candidates: int = 10, includ
         cands += [("blocked", t) for t in candidates(s)[:max_candidates]]
     if "wavefront" in schemes:
         cands.append(("wavefront", None))
+    if "overlap" in schemes and s.dtype == torch.float32 and _KIND_NAME[s.kind] != "25pt_var":
+        cands.append(("overlap", None))
     pred = [(predict(s, T, sc, t, hbm_gbs, fp_peak), sc, t) for sc, t in cands]
     pred.sort(key=lambda x: x[0])
     table, best, scale = [], (float("inf"), "plain", None), None
@@ -295,7 +307,9 @@ def tune_batch(grids: list[Stencil], T: list[int], candidates=None, reps: int = 
     Each feasible candidate is built as a Batch, captured in a CUDA graph and replayed; the
     grids advance while timing (callers reset them). Returns (tuning, table of (tuning, seconds)).
     Section II-A: the paper tunes the diamond width and thread-group size per stencil and machine;
-    here the small, uneven grids of a batch favour narrower diamonds than one large grid.
+    here the small, uneven grids of a batch favour narrower diamonds than one large grid. Batches of
+    the 7-point stencils in FP32 run overlapped tiles, which have no tuning: all candidates are
+    then the same launch, and any of those that the library accepts may be returned.
     """
     from .batch import Batch
     table = []

@@ -151,3 +151,25 @@ def test_frontline_factor_per_stencil(optin):
             assert (p(one) < p(two)) == (want == 1), (kind, cdt)
         finally:
             g.close()
+
+
+@pytest.mark.parametrize("kind,dt,cdt,offered", [
+    (C.STENCIL_7PT_CONST, torch.float32, None, True),
+    (C.STENCIL_7PT_VAR, torch.float32, torch.bfloat16, True),
+    (C.STENCIL_7PT_CONST, torch.float64, None, False),
+    (C.STENCIL_25PT_VAR, torch.float32, None, False),
+])
+def test_autotune_offers_the_overlapped_tiles_when_asked(optin, monkeypatch, kind, dt, cdt, offered):
+    """With "overlap" among the schemes, autotune times the overlapped tiles where a grid can run them and
+    keeps them where they are the fastest; other grids are tuned as without."""
+    g = HostGrid(kind, 384, 384, 384, dtype=dt, coef_dtype=cdt)
+    timed = []
+    g.set_tuning = lambda scheme, t=None: timed.append(scheme)
+    monkeypatch.setattr(tuner, "_time_run", lambda s, T, reps: {"overlap": 0.5}.get(timed[-1], 1.0))
+    try:
+        sc, tn, table = tuner.autotune(g, 50, use_cache=False, schemes=("plain", "blocked", "overlap"), max_candidates=4)
+        assert (sc == "overlap" and tn is None) == offered
+        assert any(lab == "overlap" for lab, _, _ in table) == offered
+        assert timed[-1] == sc
+    finally:
+        g.close()
