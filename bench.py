@@ -366,6 +366,17 @@ def traffic_from_profile(kernel_src_hash: str):
         return None
 
 
+def compact(x):
+    """x with every float rounded to six significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: compact(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [compact(v) for v in x]
+    return x
+
+
 def src_hash():
     h = hashlib.sha256()
     for name in ("overlap_impl.cuh", "overlap.h", "overlap.cu", "common.cuh"):
@@ -544,8 +555,10 @@ def run_ours(args):
         del host_in, host_out, pipe
         torch.cuda.empty_cache()
 
-    # roofline (algorithmic bytes per LUP: a pass of three steps reads and writes the field once)
-    bpl = 2 * 4 / 3
+    # roofline (algorithmic bytes per LUP: a pass of three steps, and one of each step that is left
+    # over, reads and writes the field once)
+    passes_per_run = T // 3 + T % 3
+    bpl = 2 * 4 * passes_per_run / T
     achieved_gbs = bpl * lups * args.steps / t_blk / 1e9  # per GPU
     fp_time = model.FP_INSTR["7pt_const"] * 2 / fp32_peak
     hbm_time = bpl / (hbm_peak * 1e9)
@@ -554,7 +567,8 @@ def run_ours(args):
     launches_per_step = max(1, launches_timed // max(1, args.steps))
     traffic = None
     if prof is not None:
-        traffic = prof[0] * lups / launches_per_step
+        # measured per LUP in passes of three steps; a pass moves the same bytes whatever its steps
+        traffic = prof[0] * 3 * passes_per_run / T * lups / launches_per_step
     if bound == "hbm":
         roof = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
                 "frac": achieved_gbs / hbm_peak, "traffic": traffic,
@@ -607,7 +621,10 @@ def run_ours(args):
                     line[key + "_error"] = repr(exc)
                 torch.cuda.empty_cache()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        # one compact line: the table per stencil and precision goes to stderr
+        if "per_stencil" in line:
+            print("per_stencil " + json.dumps(compact(line.pop("per_stencil"))), file=sys.stderr, flush=True)
+        print(json.dumps(compact(line)), flush=True)
     ranks.barrier()
     ranks.close()
     return 0
@@ -694,6 +711,8 @@ def per_stencil(device, seed, hbm_peak, fp32_peak, fp64_peak):
         bp = model.bytes_per_lup(kind, fdt, cdt, "plain")
         peak_fp = fp64_peak if fdt == "f64" else fp32_peak
         alu_glups = peak_fp / (model.FP_INSTR[kind] * 2) / 1e9
+        # the constant FP64 plain sweep leaves 4 of its 7 operations to the FP64 pipe
+        alu_plain = alu_glups * (7 / 4 if (kind, fdt) == ("7pt_const", "f64") else 1)
         s.set_tuning("plain")
         tp = timed(s, T, 2, 1) / 2
         s.set_field(u0, halo=0.0)
@@ -727,7 +746,7 @@ def per_stencil(device, seed, hbm_peak, fp32_peak, fp64_peak):
             s.set_field(u0, halo=0.0)
             s.run(T)
             err_w = sampled_oracle_error(s, kind, n, fdt, cdt, T, seed)
-        roof_p = min(hbm_peak / bp, alu_glups)
+        roof_p = min(hbm_peak / bp, alu_plain)
         roof_b = min(hbm_peak / bb, alu_glups) if bb else None
         gp = lups / tp / 1e9
         gb = lups / tb / 1e9 if tb else None
@@ -744,9 +763,9 @@ def per_stencil(device, seed, hbm_peak, fp32_peak, fp64_peak):
                           "measured_s": m_} for t, p_, m_ in tuner.last_predictions] if tun else None,
             "model_bytes_per_lup": {"plain": bp, "blocked": bb},
             "roofline_glups": {"hbm_plain": hbm_peak / bp, "hbm_blocked": hbm_peak / bb if bb else None,
-                               "alu": alu_glups},
+                               "alu": alu_glups, "alu_plain": alu_plain},
             "roofline_frac": {"plain": gp / roof_p, "blocked": gb / roof_b if gb else None,
-                              "plain_bound": "hbm" if hbm_peak / bp <= alu_glups else "alu",
+                              "plain_bound": "hbm" if hbm_peak / bp <= alu_plain else "alu",
                               "blocked_bound": ("hbm" if hbm_peak / bb <= alu_glups else "alu") if bb else None},
             "err_vs_oracle": {"plain": err_plain, "blocked": err_blk, "wavefront": err_w},
         })
