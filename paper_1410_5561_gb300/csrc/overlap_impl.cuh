@@ -18,11 +18,12 @@
 //   425 GLUP/s, BF16, kept as stored and widened at each use, 363 -> 484).
 // * Tiles overlap: a level's outermost columns / rows are wrong where the tile ends inside the
 //   domain, one more per level, so neighbouring tiles recompute 4 columns (one vector) and
-//   H - 1 rows on each side, and chunks of z recompute H planes. CTAs of a launch never wait
-//   for each other.
+//   H - 1 rows on each side, and chunks of z recompute H planes. Tiles of one pass never wait for
+//   each other.
 // * All passes of a run are one persistent launch: (pass, tile) items are popped from a counter, and
 //   a tile waits, bounded, until its 27 neighbours (itself among them) have finished the pass
-//   before. At small grids there is no launch between passes, at large ones no last wave.
+//   before. At small grids there is no launch between passes, at large ones no last wave. The steps
+//   that are left over (T % 3) are passes of one level.
 // * The per-point operations and their order are those of common.cuh, so the results are
 //   bit-identical to the plain sweep.
 //
@@ -30,7 +31,8 @@
 // shuffle per direction and row, no redundant shared-memory traffic), the diamond kernel of
 // blocked_impl.cuh 24; HBM at 3 bytes per update is the next bound (about 2100 GLUP/s). Measured,
 // 7-point constant, GLUP/s, AUTO before (diamonds) -> this: 1024^3 856 -> 1898, 512^3 727 -> 1610,
-// 256^3 394 -> 1037, 301 x 257 x 199 241 -> 861, 64^3 16 -> 64 (plain sweep: 702, 678, 511, 473, 28).
+// 256^3 394 -> 1037, 301 x 257 x 199 241 -> 861, 64^3 16 -> 64 (plain sweep: 700, 682, 544, 503, 125; the
+// rule of STENCIL_AUTO in api.cu has both sides from 64^3 to 160^3).
 // 7-point variable 384^3: FP32 200 -> 425 (HBM at 5.2 TB/s, 13 bytes per update), BF16 253 -> 484
 // (issue and latency of the widening).
 #pragma once
