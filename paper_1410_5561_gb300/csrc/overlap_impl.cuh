@@ -191,12 +191,8 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
                             z + 1, cbar + 8 * slot);
         }
     };
-    const OvRings r0{ov_uniform(ring->fs), ov_uniform(ring->cs), ov_uniform(ring->fp), ov_uniform(ring->cp),
-                     ov_uniform(ring->lost)};
-    // iteration in which a copy did not arrive in time (the results are invalid): no more copies
-    // are issued and no more waits made, in this tile and in the CTA's later ones (overlap_rings.h)
-    int lost = ov_lost_before(r0, s_begin);
-    if (threadIdx.x == 0 && lost == OV_NOT_LOST) {
+    const OvRings r0{ov_uniform(ring->fs), ov_uniform(ring->cs), ov_uniform(ring->fp), ov_uniform(ring->cp), 0};
+    if (threadIdx.x == 0) {
         for (int p = 0; p < PD; ++p)
             if (s_begin + p < zl) copy(s_begin + p, ov_slot(r0.fs, p, S::RING));
         if constexpr (NC > 0)
@@ -247,6 +243,9 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
     // coefficient slot of plane s - 1 (level 0's) and its phase, from plane cb on
     int cl = r0.cs;
     uint32_t cph = (uint32_t)r0.cp;
+    // iteration in which a copy did not arrive in time (the results are invalid): no more copies
+    // are issued and no more waits made, and the CTA walks no more tiles (overlap_rings.h)
+    int lost = OV_NOT_LOST;
     auto arrived = [&](uint32_t b, uint32_t phase, int s) {
         if (!mbar_test(b, phase) && lost == OV_NOT_LOST && !mbar_wait(b, phase, status)) lost = s;
     };
@@ -422,20 +421,17 @@ __device__ __forceinline__ void overlap_tile(const OvGrid& A, const int src, con
     if (HL < H || mode == 2) walk(std::integral_constant<int, 2>{});
     else if (mode == 1) walk(std::integral_constant<int, 1>{});
     else walk(std::integral_constant<int, 0>{});
-    if (threadIdx.x == 0) {
-        int nf = zl - s_begin, nc = ce > cb ? ce - cb : 0;
-        if (lost != OV_NOT_LOST && !r0.lost) {
-            // the copies still in flight end before the CTA goes on (bounded): the last one of every slot
-            nf = ov_issued_fields(s_begin, zl, lost, PD);
-            nc = ov_issued_coefs(cb, ce, lost, CR);
-            for (int p = max(0, nf - S::RING); p < nf; ++p)
-                mbar_wait(bar + 8 * ov_slot(r0.fs, p, S::RING), (uint32_t)ov_phase(r0.fs, r0.fp, p, S::RING), status);
-            for (int p = max(0, nc - CR); NC > 0 && p < nc; ++p)
-                mbar_wait(cbar + 8 * ov_slot(r0.cs, p, CR), (uint32_t)ov_phase(r0.cs, r0.cp, p, CR), status);
-        }
-        // read by every thread after the barrier that follows the tile
-        *ring = ov_rings_after(r0, nf, NC > 0 ? nc : 0, S::RING, CR, lost != OV_NOT_LOST);
+    if (threadIdx.x == 0 && lost != OV_NOT_LOST) {
+        ring->lost = 1;
+        // the copies still in flight end before the CTA goes on (bounded): the last one of every slot
+        const int fl = ov_last_field(s_begin, zl, lost, PD), cf = ov_last_coef(cb, ce, lost, CR);
+        for (int p = max(0, fl - S::RING + 1); p <= fl; ++p)
+            mbar_wait(bar + 8 * ov_slot(r0.fs, p, S::RING), (uint32_t)ov_phase(r0.fs, r0.fp, p, S::RING), status);
+        for (int p = max(0, cf - CR + 1); NC > 0 && p <= cf; ++p)
+            mbar_wait(cbar + 8 * ov_slot(r0.cs, p, CR), (uint32_t)ov_phase(r0.cs, r0.cp, p, CR), status);
     }
+    // read by every thread after the barrier that follows the tile
+    if (threadIdx.x == 0) ov_advance<(NC > 0)>(ring, r0, r0.fs + zl - s_begin, r0.cs + ce - cb, S::RING, CR);
 }
 
 __device__ __forceinline__ int ov_ld_acquire(const int* p) {
@@ -501,14 +497,16 @@ __global__ void __launch_bounds__(NW * 32, 1) overlap_kernel(const __grid_consta
                     fence_proxy_async_global();
                 }
             }
-            if (threadIdx.x == 0) s_item = i;
+            // (~i: published without being walked)
+            if (threadIdx.x == 0) s_item = i < items && !ov_walks(s_ring) ? ~i : i;
         }
         __syncthreads();
-        const int i = ov_uniform(s_item);
+        const int w = ov_uniform(s_item), i = w < 0 ? ~w : w;
         if (i >= items) break;
         const int p = i / tiles, t = i - p * tiles;
         const int bx = t % G.ntx, by = t / G.ntx % G.nty, bz = t / (G.ntx * G.nty), src = (G.p0 + p) & 1;
-        if (p < G.full) overlap_tile<KIND, TC, NW, RB, H, PD, CR, H, false>(G, src, bx, by, bz, s0, &s_ring, C.status);
+        if (w < 0) {
+        } else if (p < G.full) overlap_tile<KIND, TC, NW, RB, H, PD, CR, H, false>(G, src, bx, by, bz, s0, &s_ring, C.status);
         else overlap_tile<KIND, TC, NW, RB, H, PD, CR, 1, false>(G, src, bx, by, bz, s0, &s_ring, C.status);
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -576,10 +574,11 @@ __global__ void __launch_bounds__(NW * 32, 1) overlap_batch_kernel(const OvBatch
                     for (int m = 0; m < S::NC; ++m) tma_map_acquire(&G.cmap[m]);
                 }
             }
-            if (threadIdx.x == 0) s_item = i;
+            // (~i: published without being walked)
+            if (threadIdx.x == 0) s_item = i < B.nitems && !ov_walks(s_ring) ? ~i : i;
         }
         __syncthreads();
-        const int i = ov_uniform(s_item);
+        const int w = ov_uniform(s_item), i = w < 0 ? ~w : w;
         if (i >= B.nitems) break;
         const int src = ov_uniform(s_src);
         const int ig = ov_uniform(B.items[i].g), g = ig < 0 ? ~ig : ig;
@@ -587,7 +586,8 @@ __global__ void __launch_bounds__(NW * 32, 1) overlap_batch_kernel(const OvBatch
         const OvGrid& G = B.grids[g];
         const int ntx = ov_uniform(G.ntx), nty = ov_uniform(G.nty);
         const int bx = t % ntx, by = t / ntx % nty, bz = t / (ntx * nty);
-        if (p < ov_uniform(G.full)) overlap_tile<KIND, TC, NW, RB, H, PD, CR, H, true>(G, src, bx, by, bz, s0, &s_ring, C.status);
+        if (w < 0) {
+        } else if (p < ov_uniform(G.full)) overlap_tile<KIND, TC, NW, RB, H, PD, CR, H, true>(G, src, bx, by, bz, s0, &s_ring, C.status);
         else overlap_tile<KIND, TC, NW, RB, H, PD, CR, 1, true>(G, src, bx, by, bz, s0, &s_ring, C.status);
         __syncthreads();
         if (threadIdx.x == 0) {

@@ -32,9 +32,10 @@ extern "C" int walk(int PD, int CR, const int* nfs, const int* ncs, int tiles, i
     int fault = 0, lost_seen = 0;
     for (int t = 0; t < tiles; ++t) {
         const int nf = nfs[t], nc = ncs[t], base = 100000 * (t + 1), its = nf + 3;
-        int lost = ov_lost_before(r, 0);
+        if (!ov_walks(r)) continue;
+        int lost = OV_NOT_LOST;
         const int lf = t == bad && !coef ? base + late : -1, lc = t == bad && coef ? base + late : -1;
-        if (lost == OV_NOT_LOST) {
+        {
             for (int p = 0; p < PD && p < nf; ++p) F.arm(ov_slot(r.fs, p, RING), base + p);
             for (int p = 0; p < CR - 1 && p < nc; ++p) C.arm(ov_slot(r.cs, p, CR), base + p);
         }
@@ -56,10 +57,9 @@ extern "C" int walk(int PD, int CR, const int* nfs, const int* ncs, int tiles, i
             read(F, s, nf, r.fs, r.fp, RING);
             read(C, s - 1, nc, r.cs, r.cp, CR);
         }
-        int mf = nf, mc = nc;
-        if (lost != OV_NOT_LOST && !r.lost) {
-            mf = ov_issued_fields(0, nf, lost, PD);
-            mc = ov_issued_coefs(0, nc, lost, CR);
+        const OvRings r0 = r;
+        if (lost != OV_NOT_LOST) {
+            const int mf = ov_last_field(0, nf, lost, PD) + 1, mc = ov_last_coef(0, nc, lost, CR) + 1;
             // the late copy lands now: the waits for the last copy of every slot see all of them end
             for (int q = 0; q < RING; ++q) F.land(q);
             for (int q = 0; q < CR; ++q) C.land(q);
@@ -72,7 +72,8 @@ extern "C" int walk(int PD, int CR, const int* nfs, const int* ncs, int tiles, i
                 if (!C.test(q, ov_phase(r.cs, r.cp, p, CR)) || C.held[q] != base + p) fault |= 4;
             }
         }
-        r = ov_rings_after(r, mf, mc, RING, CR, lost != OV_NOT_LOST);
+        if (lost != OV_NOT_LOST) r.lost = 1;
+        ov_advance<true>(&r, r0, r0.fs + nf, r0.cs + nc, RING, CR);
         if (t > bad && bad >= 0 && lost_seen && lost == OV_NOT_LOST && after) fault |= 8;  // copied again
     }
     for (int q = 0; q < RING; ++q) fault |= F.flight[q] ? 16 : 0;
