@@ -60,6 +60,8 @@ struct CopySplit {
     int lg;
     unsigned xblocks;
     long long seg;
+    // Whether the kernels need the split: not where a CTA has COPY_WARPS whole rows.
+    bool cut() const { return lg != 3 || xblocks != 1; }
 };
 // ny rows a plane, rows in all, units a row.
 inline CopySplit copy_split(int ny, long long rows, long long units) {
