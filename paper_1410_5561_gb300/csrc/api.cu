@@ -119,8 +119,8 @@ static int check_tune(const stencil_grid* h, const BlockedTune& t) {
 // overlapped / plain: 7-point constant 2000 x 2000 x 1 222 / 424, FP32 coefficients 69 / 137, BF16 89 / 218; two
 // planes 391 / 518, 118 / 155, 153 / 244; four 619 / 548, 187 / 168, 242 / 256), fewer than 2^20 points (2000 x 31
 // x 6: 81 / 143, 83 / 120, 73 / 142), and, but for FP32 coefficients, which HBM bounds either way, rows
-// that fill few warps of a tile (2000 x 1 x 2000: 99 / 133, 71 / 42, 66 / 71; 5000 x 3 x 124 and 5000 x 6 x 201
-// 0.46 and 0.81 of the plain sweep, BF16 0.77 and 0.89; 2000 x 4 x 2000 1.18 and 1.27).
+// that fill few warps of a tile (2000 x 1 x 2000: 99 / 133, 71 / 42, 66 / 71; constant 5000 x 3 x 124 and 20000 x 3
+// x 139 0.46 and 0.72 of the plain sweep, BF16 0.77 and 1.08; 2000 x 4 x 2000 1.18 and 1.27).
 //
 // On shorter rows AUTO keeps to one launch a run, also on small grids, where the plain sweep's steps
 // have become the faster ones (T = 100 alone, overlapped / plain: 7-point constant 64^3 67 / 125, 96^3 220 / 284,
@@ -133,7 +133,7 @@ static bool auto_overlap(const stencil_grid* h) {
     const bool bf16 = h->cdt == STENCIL_BF16;
     if (L.nz <= (bf16 ? 4 : 2) || points < (1 << 20)) return false;
     if (h->kind == STENCIL_7PT_VAR && !bf16) return true;
-    return !(L.ny <= 2 || (L.ny < 8 && points < (1 << 23)));
+    return !(L.ny <= 2 || (L.ny < 8 && points < (bf16 ? 1 << 22 : 1 << 23)));
 }
 
 namespace stg {
