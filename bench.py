@@ -379,7 +379,7 @@ def compact(x):
 
 def src_hash():
     h = hashlib.sha256()
-    for name in ("overlap_impl.cuh", "overlap.h", "overlap.cu", "common.cuh"):
+    for name in ("overlap_impl.cuh", "overlap_rings.h", "overlap.h", "overlap.cu", "common.cuh"):
         with open(os.path.join(ROOT, "paper_1410_5561_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
